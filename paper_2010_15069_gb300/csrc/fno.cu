@@ -45,7 +45,8 @@ struct spgpe_fno {
   std::vector<float *> vs, us;
   std::vector<float2 *> vh;
   float *X1 = nullptr, *hp = nullptr, *h = nullptr, *dh = nullptr, *dv = nullptr, *dv2 = nullptr, *dout = nullptr;
-  float2 *oh = nullptr, *G = nullptr, *doh = nullptr;
+  float2 *oh = nullptr, *G = nullptr;
+  std::vector<float2 *> dohs;  // gradients of the mixed spectra, per layer
   float *part = nullptr;
   size_t part_n = 0;
   double *sums = nullptr;
@@ -132,12 +133,14 @@ int ensure_workspace(spgpe_fno *f, int B, int n) {
   for (float *p : f->vs) release(f, p);
   for (float *p : f->us) release(f, p);
   for (float2 *p : f->vh) release(f, p);
+  for (float2 *p : f->dohs) release(f, p);
   for (void *p : {(void *)f->X1, (void *)f->hp, (void *)f->h, (void *)f->dh, (void *)f->dv, (void *)f->dv2,
-                  (void *)f->dout, (void *)f->oh, (void *)f->G, (void *)f->doh, (void *)f->part, (void *)f->sums})
+                  (void *)f->dout, (void *)f->oh, (void *)f->G, (void *)f->part, (void *)f->sums})
     release(f, p);
   f->vs.assign(f->L + 1, nullptr);
   f->us.assign(f->L, nullptr);
   f->vh.assign(f->L, nullptr);
+  f->dohs.assign(f->L, nullptr);
   f->ws_b = f->ws_n = 0;
   const size_t P = (size_t)n * n, act = (size_t)B * f->W * P, hid = (size_t)B * f->H * P;
   const size_t spec = (size_t)B * f->W * 2 * f->M * f->M, rows = (size_t)B * f->W * n * f->M;
@@ -145,7 +148,8 @@ int ensure_workspace(spgpe_fno *f, int B, int n) {
   for (int l = 0; l <= f->L; ++l)
     if ((r = falloc(f, &f->vs[l], act))) return r;
   for (int l = 0; l < f->L; ++l)
-    if ((r = falloc(f, &f->us[l], act)) || (r = falloc(f, &f->vh[l], spec))) return r;
+    if ((r = falloc(f, &f->us[l], act)) || (r = falloc(f, &f->vh[l], spec)) || (r = falloc(f, &f->dohs[l], spec)))
+      return r;
   // split-K partials of the weight gradients: batch x splits x (largest weight)
   const int splits = (int)std::max<size_t>(1, P / 1024);
   size_t wmax = std::max<size_t>((size_t)f->W * f->cin, (size_t)f->W * f->W);
@@ -154,7 +158,7 @@ int ensure_workspace(spgpe_fno *f, int B, int n) {
   if ((r = falloc(f, &f->X1, rows * 2)) || (r = falloc(f, &f->hp, hid)) || (r = falloc(f, &f->h, hid)) ||
       (r = falloc(f, &f->dh, hid)) || (r = falloc(f, &f->dv, act)) || (r = falloc(f, &f->dv2, act)) ||
       (r = falloc(f, &f->dout, (size_t)B * f->cout * P)) || (r = falloc(f, &f->oh, spec)) ||
-      (r = falloc(f, &f->G, rows)) || (r = falloc(f, &f->doh, spec)) || (r = falloc(f, &f->part, f->part_n)) ||
+      (r = falloc(f, &f->G, rows)) || (r = falloc(f, &f->part, f->part_n)) ||
       (r = falloc(f, &f->sums, (size_t)130 * B)))
     return r;
   f->ws_b = B;
@@ -228,7 +232,7 @@ int read_flags(spgpe_fno *f) {
   return SPGPE_OK;
 }
 
-// grad[M][N] += sum_b sum_p A[b](m, p) Bm[b](p, n): split-K over the points,
+// grad[M][N] = sum_b sum_p A[b](m, p) Bm[b](p, n): split-K over the points,
 // partials reduced in a fixed order.
 int wgrad(spgpe_fno *f, int M, int N, long P, int B, const float *A, long sAb, const float *Bm, long sBn, long sBb,
           float *grad) {
@@ -241,9 +245,24 @@ int wgrad(spgpe_fno *f, int M, int N, long P, int B, const float *A, long sAb, c
   g.partial = true;
   g.sCs = (long)M * N;
   FCK(f, greal(f, g, f->st));
-  FCK(f, sum_splits(f->part, (long)M * N, B * splits, grad, true, f->st));
+  FCK(f, sum_splits(f->part, (long)M * N, B * splits, grad, false, f->st));
   return SPGPE_OK;
 }
+
+// The per-mode channel mixing of layer l (into oh): in[b][c][m] to
+// sum_c R[m][o][c] in[b][c][m], or with the conjugate transpose of R.
+cudaError_t mix_spectra(const spgpe_fno *f, int l, const float2 *in, int B, bool transposed) {
+  const long W = f->W, SP = 2L * f->M * f->M;
+  const void *R = bfp(f, f->oR[l]);
+  if (mix_applies(f->W, f->M)) return mix_modes(R, in, f->oh, f->W, f->M, B, transposed, f->st);
+  return gemm_complex(transposed ? cg(W, B, W, SP, R, true, true, 1, W, W * W, in, false, SP, W * SP, 1, f->oh, SP, W * SP, 1)
+                                 : cg(W, B, W, SP, R, true, false, W, 1, W * W, in, false, SP, W * SP, 1, f->oh, SP, W * SP, 1),
+                      f->st);
+}
+
+// Whether the spectral weights' gradient comes from (and can be applied in)
+// the one-pass kernels.
+bool fused_mix(const spgpe_fno *f, int B) { return mix_applies(f->W, f->M) && B <= kMixGradBatch; }
 
 int forward(spgpe_fno *f, const float *a, int B, int n, float *out) {
   int r;
@@ -268,9 +287,7 @@ int forward(spgpe_fno *f, const float *a, int B, int n, float *out) {
                            SP),
                         st));
     // channel mixing per mode: oh[b][o][m] = sum_c R[m][o][c] vh[b][c][m]
-    FCK(f, gemm_complex(cg(W, B, W, SP, bfp(f, f->oR[l]), true, false, W, 1, W * W, f->vh[l], false, SP, W * SP, 1,
-                           f->oh, SP, W * SP, 1),
-                        st));
+    FCK(f, mix_spectra(f, l, f->vh[l], B, false));
     // inverse along y: G = conj(Ey)^T oh per (sample, channel)
     FCK(f, gemm_complex(cg(n, M, 2 * M, B * W, f->Ey, false, true, 1, n, 0, f->oh, false, M, 1, SP, f->G, M, 1, n * M),
                         st));
@@ -309,14 +326,16 @@ int forward(spgpe_fno *f, const float *a, int B, int n, float *out) {
   return SPGPE_OK;
 }
 
-// Loss (mean relative squared error) and gradient of all parameters into f->g.
-int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, float *out, double *loss) {
+// Loss (mean relative squared error) and gradient of all parameters into f->g;
+// without spectral_grad the spectral weights' part of f->g is left alone (it
+// follows from vh and dohs).
+int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, float *out, double *loss,
+             bool spectral_grad) {
   int r = forward(f, a, B, n, out);
   if (r) return r;
   const long P = (long)n * n, W = f->W, M = f->M, H = f->H, C = f->cout;
   const long WP = W * P, SP = 2 * M * M;
   cudaStream_t st = f->st;
-  FCK(f, cudaMemsetAsync(f->g, 0, (size_t)f->nparam * sizeof(float), st));
   FCK(f, loss_terms(out, target, C * P, B, f->sums, f->dout, st));
   // output layer
   if ((r = wgrad(f, C, H, P, B, f->dout, C * P, f->h, P, H * P, f->g + f->oQ2))) return r;
@@ -348,16 +367,21 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
     // spectral part: dG = du Exi^T (into X1; as dG^T = Exi du^T), doh = Ey dG
     FCK(f, greal(f, rg(2 * M, B * W * n, n, f->Exi, false, n, 1, du, 1, n, f->X1, 1, 2 * M), st));
     const float2 *dG = reinterpret_cast<const float2 *>(f->X1);
-    FCK(f, gemm_complex(cg(2 * M, M, n, B * W, f->Ey, false, false, n, 1, 0, dG, false, M, 1, n * M, f->doh, M, 1, SP),
-                        st));
-    // dR[m] += sum_b doh[b][:, m] vh[b][:, m]^H
-    FCK(f, gemm_complex(cg(W, W, B, SP, f->doh, false, false, SP, W * SP, 1, f->vh[l], true, W * SP, SP, 1,
-                           reinterpret_cast<float2 *>(f->g + f->oR[l]), W, 1, W * W, 1.f),
+    float2 *doh = f->dohs[l];
+    FCK(f, gemm_complex(cg(2 * M, M, n, B * W, f->Ey, false, false, n, 1, 0, dG, false, M, 1, n * M, doh, M, 1, SP),
                         st));
     // dvh[b][c][m] = sum_o conj(R[m][o][c]) doh[b][o][m]  (into oh)
-    FCK(f, gemm_complex(cg(W, B, W, SP, bfp(f, f->oR[l]), true, true, 1, W, W * W, f->doh, false, SP, W * SP, 1,
-                           f->oh, SP, W * SP, 1),
-                        st));
+    FCK(f, mix_spectra(f, l, doh, B, true));
+    // dR[m] = sum_b doh[b][:, m] vh[b][:, m]^H, unless the caller takes it from the spectra
+    if (spectral_grad) {
+      if (fused_mix(f, B)) {
+        FCK(f, mix_gradient(doh, f->vh[l], f->W, f->M, B, f->g + f->oR[l], st));
+      } else {
+        FCK(f, gemm_complex(cg(W, W, B, SP, doh, false, false, SP, W * SP, 1, f->vh[l], true, W * SP, SP, 1,
+                               reinterpret_cast<float2 *>(f->g + f->oR[l]), W, 1, W * W),
+                            st));
+      }
+    }
     // dX1 = conj(Ey)^T dvh (into G), dv += dX1 Exr^T
     FCK(f, gemm_complex(cg(n, M, 2 * M, B * W, f->Ey, false, true, 1, n, 0, f->oh, false, M, 1, SP, f->G, M, 1, n * M),
                         st));
@@ -514,7 +538,7 @@ int spgpe_fno_gradient(spgpe_fno *f, const float *a, const float *target, int ba
   int r = check_shape(f, a, batch, n);
   if (r) return r;
   if (!target || !out) return ffail(f, SPGPE_EINVAL, "NULL target or output");
-  if ((r = gradient(f, a, target, batch, n, out, loss))) return r;
+  if ((r = gradient(f, a, target, batch, n, out, loss, true))) return r;
   if (grad_host) {
     FCK(f, cudaMemcpyAsync(grad_host, f->g, (size_t)f->nparam * sizeof(float), cudaMemcpyDeviceToHost, f->st));
     FCK(f, cudaStreamSynchronize(f->st));
@@ -528,9 +552,35 @@ int spgpe_fno_train_step(spgpe_fno *f, const float *a, const float *target, int 
   int r = check_shape(f, a, batch, n);
   if (r) return r;
   if (!target || !out || !(lr > 0) || !std::isfinite(lr)) return ffail(f, SPGPE_EINVAL, "bad target, output or lr");
-  if ((r = gradient(f, a, target, batch, n, out, loss))) return r;
+  // the spectral weights (nearly all parameters) take their Adam step straight
+  // from the spectra, without a gradient in memory, where the kernel applies
+  const bool fused = fused_mix(f, batch);
+  if ((r = gradient(f, a, target, batch, n, out, loss, !fused))) return r;
   ++f->t;
-  FCK(f, adam_update(f->w, f->wb, f->wr, f->g, f->m, f->v, f->nparam, (float)lr, f->t, f->st));
+  if (!fused) {
+    Ranges all;
+    all.n = 1;
+    all.begin[0] = 0;
+    all.end[0] = f->nparam;
+    FCK(f, adam_update(f->w, f->wb, f->wr, f->g, f->m, f->v, all, (float)lr, f->t, f->st));
+    return SPGPE_OK;
+  }
+  for (int l = 0; l < f->L; ++l) {
+    const long o = f->oR[l];
+    FCK(f, mix_adam(f->dohs[l], f->vh[l], f->W, f->M, batch, f->w + o, f->m + o, f->v + o,
+                    static_cast<uint16_t *>(f->wb) + o, (float)lr, f->t, f->st));
+  }
+  // what lies between the spectral weights
+  const long nR = 2L * f->M * f->M * f->W * f->W * 2;
+  Ranges rg;
+  for (int l = 0; l <= f->L; ++l) {
+    rg.begin[rg.n] = l == 0 ? 0 : f->oR[l - 1] + nR;
+    rg.end[rg.n] = l == f->L ? f->nparam : f->oR[l];
+    if (++rg.n == kRanges || l == f->L) {
+      FCK(f, adam_update(f->w, f->wb, f->wr, f->g, f->m, f->v, rg, (float)lr, f->t, f->st));
+      rg.n = 0;
+    }
+  }
   return SPGPE_OK;
 }
 

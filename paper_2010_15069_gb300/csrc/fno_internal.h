@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 namespace spgpe {
 namespace fno {
 
@@ -55,15 +57,48 @@ cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool a
 cudaError_t gemm_complex(const GemmC &g, cudaStream_t st);
 cudaError_t gelu_forward(const float *u, float *v, long n, cudaStream_t st);
 cudaError_t gelu_backward(const float *u, float *d, long n, cudaStream_t st);
-// grad[c] += sum over the batch and the points of x[b][c][p]; scratch holds
+// grad[c] = sum over the batch and the points of x[b][c][p]; scratch holds
 // 64 C doubles.
 cudaError_t bias_gradient(const float *x, int B, int C, long P, float *grad, double *scratch, cudaStream_t st);
 // sums[2 b], sums[2 b + 1] = sum (out - t)^2, sum t^2 of sample b; sums holds
 // 130 B doubles (the rest is scratch); dout (nullable) = 2 (out - t) / den_b / B.
 cudaError_t loss_terms(const float *out, const float *t, long n, int B, double *sums, float *dout, cudaStream_t st);
-// Adam on the FP32 masters w; wb (bfloat16) and wr (FP32) receive the rounded weights.
-cudaError_t adam_update(float *w, void *wb, float *wr, const float *g, float *m, float *v, long n, float lr, int t,
-                        cudaStream_t st);
+// Adam (Kingma & Ba 2015) with bias correction: the rates of step t (from 1),
+// and one parameter's update.
+struct AdamRates {
+  float lr = 0.f, c1 = 1.f, c2 = 1.f;
+};
+inline AdamRates adam_rates(float lr, int t) {
+  return {lr, (float)(1.0 - std::pow(0.9, t)), (float)(1.0 - std::pow(0.999, t))};
+}
+__device__ __forceinline__ void adam_one(float &w, float &m, float &v, float g, const AdamRates &r) {
+  m = fmaf(0.9f, m, 0.1f * g);
+  v = fmaf(0.999f, v, 0.001f * g * g);
+  w -= r.lr * (m / r.c1) / (sqrtf(v / r.c2) + 1e-8f);
+}
+// Up to kRanges [begin, end) ranges of the parameter vector.
+constexpr int kRanges = 16;
+struct Ranges {
+  int n = 0;
+  long begin[kRanges], end[kRanges];
+};
+// Adam on the FP32 masters w of the ranges; wb (bfloat16) and wr (FP32)
+// receive the rounded weights.
+cudaError_t adam_update(float *w, void *wb, float *wr, const float *g, float *m, float *v, const Ranges &rg, float lr,
+                        int t, cudaStream_t st);
+// The spectral layers' channel mixing per mode (fno_mix.cu; W = 32 or 64
+// channels, a multiple of 8 modes, bfloat16 pairs R[mode][o][c], spectra
+// [sample][channel][mode]): out[b][o][m] = sum_c R[m][o][c] in[b][c][m], or
+// transposed out[b][c][m] = sum_o conj(R[m][o][c]) in[b][o][m]; the weights'
+// gradient dR[m][o][c] = sum_b d[b][o][m] conj(v[b][c][m]) for at most
+// kMixGradBatch samples, written to g or applied as their Adam step.
+constexpr int kMixGradBatch = 8;
+bool mix_applies(int width, int modes);
+cudaError_t mix_modes(const void *R, const float2 *in, float2 *out, int width, int modes, int batch, bool transposed,
+                      cudaStream_t st);
+cudaError_t mix_gradient(const float2 *d, const float2 *v, int width, int modes, int batch, float *g, cudaStream_t st);
+cudaError_t mix_adam(const float2 *d, const float2 *v, int width, int modes, int batch, float *w, float *m, float *ve,
+                     void *wb, float lr, int t, cudaStream_t st);
 cudaError_t round_weights(const float *w, void *wb, float *wr, long n, cudaStream_t st);
 
 }  // namespace fno

@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "fno_internal.h"
@@ -300,8 +301,7 @@ __global__ void gelu_bwd(const float *__restrict__ u, float *__restrict__ d, lon
     d[i] *= gelu_d(u[i]);
 }
 
-// grad[c] (+)= sum over samples b and points p of x[b][c][p] (fixed order).
-// Bias gradient grad[c] += sum_b sum_p x[b][c][p], in two stages: kBiasSlices
+// Bias gradient grad[c] = sum_b sum_p x[b][c][p], in two stages: kBiasSlices
 // blocks per channel each sum a contiguous slice of the points (float32 per
 // thread over at most a few dozen values, then a fixed tree), and one block
 // adds the slices of every channel in a fixed order in FP64.
@@ -333,7 +333,7 @@ __global__ void bias_grad_sum(const double *__restrict__ part, int C, float *gra
   for (int c = threadIdx.x; c < C; c += blockDim.x) {
     double t = 0.0;
     for (int sl = 0; sl < kBiasSlices; ++sl) t += part[(long)c * kBiasSlices + sl];
-    grad[c] += (float)t;
+    grad[c] = (float)t;
   }
 }
 
@@ -395,16 +395,17 @@ __global__ void loss_grad(const float *__restrict__ out, const float *__restrict
   }
 }
 
-// Adam (Kingma & Ba 2015) with bias correction on the FP32 master weights;
-// the bfloat16 weights used in the products are the rounded masters.
-__global__ void adam(float *w, __nv_bfloat16 *wb, float *wr, const float *__restrict__ g, float *m, float *v, long n,
-                     float lr, float c1, float c2) {
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = fmaf(0.9f, m[i], 0.1f * gi), vi = fmaf(0.999f, v[i], 0.001f * gi * gi);
+// Adam on the FP32 master weights of the ranges (one per gridDim.y); the
+// bfloat16 weights used in the products are the rounded masters.
+__global__ void adam(float *w, __nv_bfloat16 *wb, float *wr, const float *__restrict__ g, float *m, float *v, Ranges rg,
+                     AdamRates ar) {
+  const long e = rg.end[blockIdx.y];
+  for (long i = rg.begin[blockIdx.y] + (long)blockIdx.x * blockDim.x + threadIdx.x; i < e;
+       i += (long)gridDim.x * blockDim.x) {
+    float wi = w[i], mi = m[i], vi = v[i];
+    adam_one(wi, mi, vi, g[i], ar);
     m[i] = mi;
     v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
     w[i] = wi;
     const __nv_bfloat16 r = __float2bfloat16_rn(wi);
     wb[i] = r;
@@ -505,10 +506,13 @@ cudaError_t loss_terms(const float *out, const float *t, long n, int B, double *
   return cudaGetLastError();
 }
 
-cudaError_t adam_update(float *w, void *wb, float *wr, const float *g, float *m, float *v, long n, float lr, int t,
-                        cudaStream_t st) {
-  const float c1 = (float)(1.0 - std::pow(0.9, t)), c2 = (float)(1.0 - std::pow(0.999, t));
-  adam<<<grid_for(n), 256, 0, st>>>(w, static_cast<__nv_bfloat16 *>(wb), wr, g, m, v, n, lr, c1, c2);
+cudaError_t adam_update(float *w, void *wb, float *wr, const float *g, float *m, float *v, const Ranges &rg, float lr,
+                        int t, cudaStream_t st) {
+  long most = 0;
+  for (int i = 0; i < rg.n; ++i) most = std::max(most, rg.end[i] - rg.begin[i]);
+  if (most < 1) return cudaSuccess;
+  adam<<<dim3(grid_for(most), rg.n), 256, 0, st>>>(w, static_cast<__nv_bfloat16 *>(wb), wr, g, m, v, rg,
+                                                    adam_rates(lr, t));
   return cudaGetLastError();
 }
 
