@@ -40,6 +40,9 @@ struct spgpe_fno {
   int tw_n = 0;
   float *Exr = nullptr, *Exi = nullptr;
   float2 *Ey = nullptr;
+  uint16_t *tab[3] = {};  // tensor-core transforms' tables, by DftTable
+  float *sin32 = nullptr;
+  int sms = 0;
   // workspace for (ws_b, ws_n)
   int ws_b = 0, ws_n = 0;
   std::vector<float *> vs, us;
@@ -95,10 +98,13 @@ void release(spgpe_fno *f, void *p) {
 // Ey[j][y] = exp(-2 pi i ky_j y / n), ky_j = j (j < M) or n - 2M + j (forward along y);
 // Exi[2k][x], Exi[2k+1][x] = g_k cos, -g_k sin(2 pi k x / n) / n^2 (real part of
 // the inverse along x, g_0 = 1, g_k = 2).
+bool use_dft(const spgpe_fno *f, int n) { return f->tensor_cores && f->sms > 0 && dft_applies(n, f->M, f->W); }
+
 int ensure_twiddles(spgpe_fno *f, int n) {
   if (f->tw_n == n) return SPGPE_OK;
   const int M = f->M;
-  for (void *p : {(void *)f->Exr, (void *)f->Exi, (void *)f->Ey}) release(f, p);
+  for (void *p : {(void *)f->Exr, (void *)f->Exi, (void *)f->Ey, (void *)f->sin32}) release(f, p);
+  for (uint16_t *p : f->tab) release(f, p);
   f->tw_n = 0;
   std::vector<float> exr((size_t)n * 2 * M), exi((size_t)2 * M * n), ey((size_t)2 * M * n * 2);
   for (int x = 0; x < n; ++x)
@@ -124,6 +130,17 @@ int ensure_twiddles(spgpe_fno *f, int n) {
   FCK(f, cudaMemcpy(f->Exr, exr.data(), exr.size() * sizeof(float), cudaMemcpyHostToDevice));
   FCK(f, cudaMemcpy(f->Exi, exi.data(), exi.size() * sizeof(float), cudaMemcpyHostToDevice));
   FCK(f, cudaMemcpy(f->Ey, ey.data(), ey.size() * sizeof(float), cudaMemcpyHostToDevice));
+  if (use_dft(f, n)) {
+    for (int i = 0; i < 3; ++i) {
+      const std::vector<uint16_t> t = dft_table(static_cast<DftTable>(i), n, M);
+      if ((r = falloc(f, &f->tab[i], t.size()))) return r;
+      FCK(f, cudaMemcpy(f->tab[i], t.data(), t.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
+    }
+    std::vector<float> s32((size_t)n);
+    for (int y = 0; y < n; ++y) s32[(size_t)y] = (float)std::sin(kTwoPi * (double)(32l * y % n) / n);
+    if ((r = falloc(f, &f->sin32, s32.size()))) return r;
+    FCK(f, cudaMemcpy(f->sin32, s32.data(), s32.size() * sizeof(float), cudaMemcpyHostToDevice));
+  }
   f->tw_n = n;
   return SPGPE_OK;
 }
@@ -264,11 +281,44 @@ cudaError_t mix_spectra(const spgpe_fno *f, int l, const float2 *in, int B, bool
 // the one-pass kernels.
 bool fused_mix(const spgpe_fno *f, int B) { return mix_applies(f->W, f->M) && B <= kMixGradBatch; }
 
+// The kept modes of v [B][W][n][n] along x (with Exr, or Exi^T for the adjoint
+// of the inverse) and y: vh [B][W][2M][M].
+int spectrum(spgpe_fno *f, const float *v, bool adjoint, int B, int n, float2 *vh) {
+  const long W = f->W, M = f->M, SP = 2 * M * M;
+  if (use_dft(f, n)) {
+    FCK(f, dft_x(v, f->tab[(int)DftTable::X], adjoint, f->X1, (int)(B * W), n, f->M, f->sms, f->d_flags, f->st));
+    FCK(f, dft_y(f->X1, f->tab[(int)DftTable::Y], vh, (int)(B * W), n, f->M, f->sms, f->d_flags, f->st));
+    return SPGPE_OK;
+  }
+  // X1 = v Exr, computed as X1^T = Exr^T v^T (the long side as N)
+  if (adjoint)
+    FCK(f, greal(f, rg(2 * M, B * W * n, n, f->Exi, false, n, 1, v, 1, n, f->X1, 1, 2 * M), f->st));
+  else
+    FCK(f, greal(f, rg(2 * M, B * W * n, n, f->Exr, false, 1, 2 * M, v, 1, n, f->X1, 1, 2 * M), f->st));
+  // vh = Ey X1 per (sample, channel)
+  FCK(f, gemm_complex(cg(2 * M, M, n, B * W, f->Ey, false, false, n, 1, 0, reinterpret_cast<const float2 *>(f->X1),
+                         false, M, 1, n * M, vh, M, 1, SP),
+                      f->st));
+  return SPGPE_OK;
+}
+
+// G = conj(Ey)^T oh per (sample, channel).
+int inverse_y(spgpe_fno *f, int B, int n) {
+  const long W = f->W, M = f->M, SP = 2 * M * M;
+  if (use_dft(f, n)) {
+    FCK(f, idft_y(f->oh, f->tab[(int)DftTable::InverseY], f->sin32, f->G, (int)(B * W), n, f->M, f->d_flags, f->st));
+    return SPGPE_OK;
+  }
+  FCK(f, gemm_complex(cg(n, M, 2 * M, B * W, f->Ey, false, true, 1, n, 0, f->oh, false, M, 1, SP, f->G, M, 1, n * M),
+                      f->st));
+  return SPGPE_OK;
+}
+
 int forward(spgpe_fno *f, const float *a, int B, int n, float *out) {
   int r;
   if ((r = ensure_twiddles(f, n)) || (r = ensure_workspace(f, B, n))) return r;
   const long P = (long)n * n, W = f->W, M = f->M, H = f->H;
-  const long WP = W * P, SP = 2 * M * M;
+  const long WP = W * P;
   cudaStream_t st = f->st;
   // lift: v0 = P a + p
   GemmR g = rg(W, P, f->cin, bfp(f, f->oP), true, f->cin, 1, a, P, 1, f->vs[0], P, 1);
@@ -279,18 +329,9 @@ int forward(spgpe_fno *f, const float *a, int B, int n, float *out) {
   FCK(f, greal(f, g, st));
   for (int l = 0; l < f->L; ++l) {
     float *v = f->vs[l], *u = f->us[l];
-    // along x: X1 = v Exr, computed as X1^T = Exr^T v^T (the long side as N)
-    FCK(f, greal(f, rg(2 * M, B * W * n, n, f->Exr, false, 1, 2 * M, v, 1, n, f->X1, 1, 2 * M), st));
-    const float2 *X1c = reinterpret_cast<const float2 *>(f->X1);
-    // along y: vh = Ey X1 per (sample, channel)
-    FCK(f, gemm_complex(cg(2 * M, M, n, B * W, f->Ey, false, false, n, 1, 0, X1c, false, M, 1, n * M, f->vh[l], M, 1,
-                           SP),
-                        st));
-    // channel mixing per mode: oh[b][o][m] = sum_c R[m][o][c] vh[b][c][m]
+    if ((r = spectrum(f, v, false, B, n, f->vh[l]))) return r;
     FCK(f, mix_spectra(f, l, f->vh[l], B, false));
-    // inverse along y: G = conj(Ey)^T oh per (sample, channel)
-    FCK(f, gemm_complex(cg(n, M, 2 * M, B * W, f->Ey, false, true, 1, n, 0, f->oh, false, M, 1, SP, f->G, M, 1, n * M),
-                        st));
+    if ((r = inverse_y(f, B, n))) return r;
     // real part of the inverse along x: u = G Exi
     FCK(f, greal(f, rg(B * W * n, n, 2 * M, reinterpret_cast<const float *>(f->G), false, 2 * M, 1, f->Exi, n, 1,
                         u, n, 1),
@@ -364,12 +405,9 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
     g.sBb = WP;
     g.sCb = WP;
     FCK(f, greal(f, g, st));
-    // spectral part: dG = du Exi^T (into X1; as dG^T = Exi du^T), doh = Ey dG
-    FCK(f, greal(f, rg(2 * M, B * W * n, n, f->Exi, false, n, 1, du, 1, n, f->X1, 1, 2 * M), st));
-    const float2 *dG = reinterpret_cast<const float2 *>(f->X1);
+    // spectral part: doh = Ey (du Exi^T)
     float2 *doh = f->dohs[l];
-    FCK(f, gemm_complex(cg(2 * M, M, n, B * W, f->Ey, false, false, n, 1, 0, dG, false, M, 1, n * M, doh, M, 1, SP),
-                        st));
+    if ((r = spectrum(f, du, true, B, n, doh))) return r;
     // dvh[b][c][m] = sum_o conj(R[m][o][c]) doh[b][o][m]  (into oh)
     FCK(f, mix_spectra(f, l, doh, B, true));
     // dR[m] = sum_b doh[b][:, m] vh[b][:, m]^H, unless the caller takes it from the spectra
@@ -383,8 +421,7 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
       }
     }
     // dX1 = conj(Ey)^T dvh (into G), dv += dX1 Exr^T
-    FCK(f, gemm_complex(cg(n, M, 2 * M, B * W, f->Ey, false, true, 1, n, 0, f->oh, false, M, 1, SP, f->G, M, 1, n * M),
-                        st));
+    if ((r = inverse_y(f, B, n))) return r;
     g = rg(B * W * n, n, 2 * M, reinterpret_cast<const float *>(f->G), false, 2 * M, 1, f->Exr, 1, 2 * M, dvn, n, 1);
     g.beta = 1.f;
     FCK(f, greal(f, g, st));
@@ -488,6 +525,12 @@ int spgpe_fno_create(spgpe_fno **out, int cin, int cout, int width, int modes, i
     return r;
   }
   if (cudaMemset(f->d_flags, 0, sizeof(int)) != cudaSuccess) {
+    spgpe_fno_destroy(f);
+    return SPGPE_ECUDA;
+  }
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     spgpe_fno_destroy(f);
     return SPGPE_ECUDA;
   }

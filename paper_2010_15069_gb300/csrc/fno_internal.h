@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
+#include <vector>
 
 namespace spgpe {
 namespace fno {
@@ -55,6 +57,22 @@ bool gemm_tc_applies(const GemmR &g);
 cudaError_t gemm_real_tc(const GemmR &g, cudaStream_t st);
 cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool accumulate, cudaStream_t st);
 cudaError_t gemm_complex(const GemmC &g, cudaStream_t st);
+// Truncated Fourier transforms on the tensor cores (fno_dft.cu) of `images` n x n
+// fields with the kept modes kx < M, ky = -M .. M - 1 (M even, at most 32; n a
+// multiple of 64; `width` channels per sample, whose rows fill whole tiles of 128):
+// along x (cos, -sin; adjoint: times g_k / n^2, g_0 = 1, g_k = 2), along y, and
+// the inverse along y.
+// Tables: dft_table on the host, uploaded as they are; sin32[y] = sin(2 pi 32
+// y / n).  flags receives a wait that ran out.
+enum class DftTable { X, Y, InverseY };
+bool dft_applies(int n, int modes, int width);
+std::vector<uint16_t> dft_table(DftTable which, int n, int modes);
+cudaError_t dft_x(const float *v, const void *table, bool adjoint, float *X1, int images, int n, int modes, int sms,
+                  int *flags, cudaStream_t st);
+cudaError_t dft_y(const float *X1, const void *table, float2 *vh, int images, int n, int modes, int sms, int *flags,
+                  cudaStream_t st);
+cudaError_t idft_y(const float2 *oh, const void *table, const float *sin32, float2 *G, int images, int n, int modes,
+                   int *flags, cudaStream_t st);
 cudaError_t gelu_forward(const float *u, float *v, long n, cudaStream_t st);
 cudaError_t gelu_backward(const float *u, float *d, long n, cudaStream_t st);
 // grad[c] = sum over the batch and the points of x[b][c][p]; scratch holds
