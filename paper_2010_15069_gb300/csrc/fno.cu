@@ -40,7 +40,7 @@ struct spgpe_fno {
   int tw_n = 0;
   float *Exr = nullptr, *Exi = nullptr;
   float2 *Ey = nullptr;
-  uint16_t *tab[3] = {};  // tensor-core transforms' tables, by DftTable
+  uint16_t *tab[4] = {};  // tensor-core transforms' tables, by DftTable
   float *sin32 = nullptr;
   int sms = 0;
   // workspace for (ws_b, ws_n)
@@ -131,7 +131,7 @@ int ensure_twiddles(spgpe_fno *f, int n) {
   FCK(f, cudaMemcpy(f->Exi, exi.data(), exi.size() * sizeof(float), cudaMemcpyHostToDevice));
   FCK(f, cudaMemcpy(f->Ey, ey.data(), ey.size() * sizeof(float), cudaMemcpyHostToDevice));
   if (use_dft(f, n)) {
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < 4; ++i) {
       const std::vector<uint16_t> t = dft_table(static_cast<DftTable>(i), n, M);
       if ((r = falloc(f, &f->tab[i], t.size()))) return r;
       FCK(f, cudaMemcpy(f->tab[i], t.data(), t.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
@@ -281,6 +281,8 @@ cudaError_t mix_spectra(const spgpe_fno *f, int l, const float2 *in, int B, bool
 // the one-pass kernels.
 bool fused_mix(const spgpe_fno *f, int B) { return mix_applies(f->W, f->M) && B <= kMixGradBatch; }
 
+bool use_layer(const spgpe_fno *f, int n) { return use_dft(f, n) && layer_applies(n, f->M, f->W); }
+
 // The kept modes of v [B][W][n][n] along x (with Exr, or Exi^T for the adjoint
 // of the inverse) and y: vh [B][W][2M][M].
 int spectrum(spgpe_fno *f, const float *v, bool adjoint, int B, int n, float2 *vh) {
@@ -314,7 +316,8 @@ int inverse_y(spgpe_fno *f, int B, int n) {
   return SPGPE_OK;
 }
 
-int forward(spgpe_fno *f, const float *a, int B, int n, float *out) {
+// keep: the activations that the backward pass reads are written too.
+int forward(spgpe_fno *f, const float *a, int B, int n, float *out, bool keep) {
   int r;
   if ((r = ensure_twiddles(f, n)) || (r = ensure_workspace(f, B, n))) return r;
   const long P = (long)n * n, W = f->W, M = f->M, H = f->H;
@@ -332,6 +335,12 @@ int forward(spgpe_fno *f, const float *a, int B, int n, float *out) {
     if ((r = spectrum(f, v, false, B, n, f->vh[l]))) return r;
     FCK(f, mix_spectra(f, l, f->vh[l], B, false));
     if ((r = inverse_y(f, B, n))) return r;
+    const bool last = l == f->L - 1;
+    if (use_layer(f, n)) {
+      FCK(f, layer_forward(v, f->G, f->tab[(int)DftTable::LayerX], bfp(f, f->oW[l]), f->wr + f->ow[l],
+                           keep ? u : nullptr, f->vs[l + 1], !last, B, (int)W, n, f->M, f->sms, f->d_flags, st));
+      continue;
+    }
     // real part of the inverse along x: u = G Exi
     FCK(f, greal(f, rg(B * W * n, n, 2 * M, reinterpret_cast<const float *>(f->G), false, 2 * M, 1, f->Exi, n, 1,
                         u, n, 1),
@@ -344,7 +353,7 @@ int forward(spgpe_fno *f, const float *a, int B, int n, float *out) {
     g.beta = 1.f;
     g.bias = f->wr + f->ow[l];
     FCK(f, greal(f, g, st));
-    if (l < f->L - 1) {
+    if (!last) {
       FCK(f, gelu_forward(u, f->vs[l + 1], (long)B * WP, st));
     } else {
       FCK(f, cudaMemcpyAsync(f->vs[l + 1], u, (size_t)B * WP * sizeof(float), cudaMemcpyDeviceToDevice, st));
@@ -372,7 +381,7 @@ int forward(spgpe_fno *f, const float *a, int B, int n, float *out) {
 // follows from vh and dohs).
 int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, float *out, double *loss,
              bool spectral_grad) {
-  int r = forward(f, a, B, n, out);
+  int r = forward(f, a, B, n, out, true);
   if (r) return r;
   const long P = (long)n * n, W = f->W, M = f->M, H = f->H, C = f->cout;
   const long WP = W * P, SP = 2 * M * M;
@@ -396,15 +405,10 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
   FCK(f, greal(f, g, st));
   float *du = f->dv, *dvn = f->dv2;
   for (int l = f->L - 1; l >= 0; --l) {
-    if (l < f->L - 1) FCK(f, gelu_backward(f->us[l], du, (long)B * WP, st));
+    // (the fused layer pass has multiplied du by the activation's derivative)
+    if (l < f->L - 1 && !use_layer(f, n)) FCK(f, gelu_backward(f->us[l], du, (long)B * WP, st));
     if ((r = wgrad(f, W, W, P, B, du, WP, f->vs[l], P, WP, f->g + f->oW[l]))) return r;
     FCK(f, bias_gradient(du, B, W, P, f->g + f->ow[l], f->bscr, st));
-    // dv = W_l^T du
-    g = rg(W, P, W, bfp(f, f->oW[l]), true, 1, W, du, P, 1, dvn, P, 1);
-    g.batch = B;
-    g.sBb = WP;
-    g.sCb = WP;
-    FCK(f, greal(f, g, st));
     // spectral part: doh = Ey (du Exi^T)
     float2 *doh = f->dohs[l];
     if ((r = spectrum(f, du, true, B, n, doh))) return r;
@@ -422,6 +426,18 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
     }
     // dX1 = conj(Ey)^T dvh (into G), dv += dX1 Exr^T
     if ((r = inverse_y(f, B, n))) return r;
+    if (use_layer(f, n)) {
+      FCK(f, layer_backward(du, f->G, f->tab[(int)DftTable::LayerX], bfp(f, f->oW[l]), l > 0 ? f->us[l - 1] : nullptr,
+                            dvn, B, (int)W, n, f->M, f->sms, f->d_flags, st));
+      std::swap(du, dvn);
+      continue;
+    }
+    // dv = W_l^T du
+    g = rg(W, P, W, bfp(f, f->oW[l]), true, 1, W, du, P, 1, dvn, P, 1);
+    g.batch = B;
+    g.sBb = WP;
+    g.sCb = WP;
+    FCK(f, greal(f, g, st));
     g = rg(B * W * n, n, 2 * M, reinterpret_cast<const float *>(f->G), false, 2 * M, 1, f->Exr, 1, 2 * M, dvn, n, 1);
     g.beta = 1.f;
     FCK(f, greal(f, g, st));
@@ -573,7 +589,7 @@ int spgpe_fno_forward(spgpe_fno *f, const float *a, int batch, int n, float *out
   int r = check_shape(f, a, batch, n);
   if (r) return r;
   if (!out) return ffail(f, SPGPE_EINVAL, "NULL output");
-  return forward(f, a, batch, n, out);
+  return forward(f, a, batch, n, out, false);
 }
 
 int spgpe_fno_gradient(spgpe_fno *f, const float *a, const float *target, int batch, int n, float *out,

@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(kThreads, 1) dft(const DftArgs a) {
   }
 
   // The thread's part of a block: two runs of 8 k.  Along x: rows (tid >> 3) +
-  // 64 i, run tid & 7; along y: row tid & 127, runs (tid >> 7) + 4 i.
+  // 64 i, run tid & 7, in the order of x_slot (4 of the block's first 32 k and 4
+  // of the others, so that 8 lanes read whole 128-byte lines); along y: row tid & 127, runs (tid >> 7) + 4 i.
   float x[NB][16], c[2];
   auto load = [&](int u, int kc) {
     const int tile = tile_of(u), kb = (u / mytiles) * NB + kc;
@@ -124,8 +125,8 @@ __global__ void __launch_bounds__(kThreads, 1) dft(const DftArgs a) {
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const float4 *p = reinterpret_cast<const float4 *>(
-            a.src + (long)(tile * kTcRows + (tid >> 3) + 64 * i) * a.n + kb * kKBlock + (tid & 7) * 8);
-        const float4 v = p[0], w = p[1];
+            a.src + (long)(tile * kTcRows + (tid >> 3) + 64 * i) * a.n + kb * kKBlock + (tid & 7) * 4);
+        const float4 v = p[0], w = p[8];
         x[kc][8 * i] = v.x; x[kc][8 * i + 1] = v.y; x[kc][8 * i + 2] = v.z; x[kc][8 * i + 3] = v.w;
         x[kc][8 * i + 4] = w.x; x[kc][8 * i + 5] = w.y; x[kc][8 * i + 6] = w.z; x[kc][8 * i + 7] = w.w;
       }
@@ -500,6 +501,13 @@ bool dft_applies(int n, int modes, int width) {
 
 // (The twiddles are the float32 ones of the general path, so that both paths
 // compute the same transform.)
+// Slot of x in its 64-wide block: run r = slot / 8 holds x = 4 r .. 4 r + 3 and
+// 32 + 4 r .. 32 + 4 r + 3.
+static int x_slot(int x) {
+  const int k = x % kKBlock;
+  return 8 * ((k % 32) / 4) + k % 4 + (k >= 32 ? 4 : 0);
+}
+
 std::vector<uint16_t> dft_table(DftTable which, int n, int M) {
   if (which == DftTable::X) {  // columns 2k, 2k + 1 = cos, -sin(2 pi k x / n), k < M
     const int N = pad16(2 * M);
@@ -508,8 +516,8 @@ std::vector<uint16_t> dft_table(DftTable which, int n, int M) {
       for (int k = 0; k < M; ++k) {
         const double th = kTwoPi * (double)((long)k * x % n) / n;
         uint16_t *b = t.data() + (size_t)(x / kKBlock) * 3 * N * kKBlock;
-        put3(b, N, 2 * k, x % kKBlock, (float)std::cos(th));
-        put3(b, N, 2 * k + 1, x % kKBlock, (float)-std::sin(th));
+        put3(b, N, 2 * k, x_slot(x), (float)std::cos(th));
+        put3(b, N, 2 * k + 1, x_slot(x), (float)-std::sin(th));
       }
     return t;
   }
@@ -522,6 +530,17 @@ std::vector<uint16_t> dft_table(DftTable which, int n, int M) {
         uint16_t *b = t.data() + (size_t)(y / kKBlock) * 3 * N * kKBlock;
         put3(b, N, 2 * k, y % kKBlock, (float)std::cos(th));
         put3(b, N, 2 * k + 1, y % kKBlock, (float)std::sin(th));
+      }
+    return t;
+  }
+  if (which == DftTable::LayerX) {  // row x, slots 2k, 2k + 1 = cos, -sin(2 pi k x / n), k < M; tiles of 128 rows
+    std::vector<uint16_t> t((size_t)((n + kTcRows - 1) / kTcRows) * 3 * kTcRows * kKBlock, 0);
+    for (int x = 0; x < n; ++x)
+      for (int k = 0; k < M; ++k) {
+        const double th = kTwoPi * (double)((long)k * x % n) / n;
+        uint16_t *b = t.data() + (size_t)(x / kTcRows) * 3 * kTcRows * kKBlock;
+        put3(b, kTcRows, x % kTcRows, 2 * k, (float)std::cos(th));
+        put3(b, kTcRows, x % kTcRows, 2 * k + 1, (float)-std::sin(th));
       }
     return t;
   }

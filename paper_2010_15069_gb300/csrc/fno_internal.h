@@ -64,7 +64,7 @@ cudaError_t gemm_complex(const GemmC &g, cudaStream_t st);
 // the inverse along y.
 // Tables: dft_table on the host, uploaded as they are; sin32[y] = sin(2 pi 32
 // y / n).  flags receives a wait that ran out.
-enum class DftTable { X, Y, InverseY };
+enum class DftTable { X, Y, InverseY, LayerX };
 bool dft_applies(int n, int modes, int width);
 std::vector<uint16_t> dft_table(DftTable which, int n, int modes);
 cudaError_t dft_x(const float *v, const void *table, bool adjoint, float *X1, int images, int n, int modes, int sms,
@@ -73,6 +73,17 @@ cudaError_t dft_y(const float *X1, const void *table, float2 *vh, int images, in
                   cudaStream_t st);
 cudaError_t idft_y(const float2 *oh, const void *table, const float *sin32, float2 *G, int images, int n, int modes,
                    int *flags, cudaStream_t st);
+// The rest of a spectral layer in one pass (fno_layer.cu; W = 32 or 64 where
+// dft_applies): forward, u = W v + w + the real inverse of G along x, written
+// to u (null: not kept) with out = gelu(u), or (activate false) out = u;
+// backward, out = (W^T du + the adjoint of the transform along x of G) times
+// gelu'(u_prev) (null: without).  table: dft_table(LayerX).
+bool layer_applies(int n, int modes, int width);
+cudaError_t layer_forward(const float *v, const float2 *G, const void *table, const void *weights, const float *bias,
+                          float *u, float *out, bool activate, int batch, int width, int n, int modes, int sms,
+                          int *flags, cudaStream_t st);
+cudaError_t layer_backward(const float *du, const float2 *G, const void *table, const void *weights, const float *u_prev,
+                           float *out, int batch, int width, int n, int modes, int sms, int *flags, cudaStream_t st);
 cudaError_t gelu_forward(const float *u, float *v, long n, cudaStream_t st);
 cudaError_t gelu_backward(const float *u, float *d, long n, cudaStream_t st);
 // grad[c] = sum over the batch and the points of x[b][c][p]; scratch holds
@@ -93,6 +104,11 @@ __device__ __forceinline__ void adam_one(float &w, float &m, float &v, float g, 
   m = fmaf(0.9f, m, 0.1f * g);
   v = fmaf(0.999f, v, 0.001f * g * g);
   w -= r.lr * (m / r.c1) / (sqrtf(v / r.c2) + 1e-8f);
+}
+// The exact GELU x Phi(x) and its derivative.
+__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
+__device__ __forceinline__ float gelu_d(float x) {
+  return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
 }
 // Up to kRanges [begin, end) ranges of the parameter vector.
 constexpr int kRanges = 16;

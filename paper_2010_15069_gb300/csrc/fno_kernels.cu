@@ -286,11 +286,6 @@ __global__ void __launch_bounds__(256) gemm_c(int M, int N, int K, const TA *__r
   }
 }
 
-__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_d(float x) {
-  return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
-}
-
 __global__ void gelu_fwd(const float *__restrict__ u, float *__restrict__ v, long n) {
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
     v[i] = gelu_f(u[i]);
