@@ -40,8 +40,9 @@ struct spgpe_fno {
   int tw_n = 0;
   float *Exr = nullptr, *Exi = nullptr;
   float2 *Ey = nullptr;
-  uint16_t *tab[4] = {};  // tensor-core transforms' tables, by DftTable
+  uint16_t *tab[2] = {};  // tensor-core transforms' tables, by DftTable
   float *sin32 = nullptr;
+  float2 *EyT = nullptr;  // Ey by y: [y][j]
   int sms = 0;
   // workspace for (ws_b, ws_n)
   int ws_b = 0, ws_n = 0;
@@ -103,7 +104,7 @@ bool use_dft(const spgpe_fno *f, int n) { return f->tensor_cores && f->sms > 0 &
 int ensure_twiddles(spgpe_fno *f, int n) {
   if (f->tw_n == n) return SPGPE_OK;
   const int M = f->M;
-  for (void *p : {(void *)f->Exr, (void *)f->Exi, (void *)f->Ey, (void *)f->sin32}) release(f, p);
+  for (void *p : {(void *)f->Exr, (void *)f->Exi, (void *)f->Ey, (void *)f->sin32, (void *)f->EyT}) release(f, p);
   for (uint16_t *p : f->tab) release(f, p);
   f->tw_n = 0;
   std::vector<float> exr((size_t)n * 2 * M), exi((size_t)2 * M * n), ey((size_t)2 * M * n * 2);
@@ -131,11 +132,17 @@ int ensure_twiddles(spgpe_fno *f, int n) {
   FCK(f, cudaMemcpy(f->Exi, exi.data(), exi.size() * sizeof(float), cudaMemcpyHostToDevice));
   FCK(f, cudaMemcpy(f->Ey, ey.data(), ey.size() * sizeof(float), cudaMemcpyHostToDevice));
   if (use_dft(f, n)) {
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 2; ++i) {
       const std::vector<uint16_t> t = dft_table(static_cast<DftTable>(i), n, M);
       if ((r = falloc(f, &f->tab[i], t.size()))) return r;
       FCK(f, cudaMemcpy(f->tab[i], t.data(), t.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
     }
+    std::vector<float> eyt(ey.size());
+    for (int j = 0; j < 2 * M; ++j)
+      for (int y = 0; y < n; ++y)
+        for (int c = 0; c < 2; ++c) eyt[((size_t)y * 2 * M + j) * 2 + c] = ey[((size_t)j * n + y) * 2 + c];
+    if ((r = falloc(f, &f->EyT, (size_t)2 * M * n))) return r;
+    FCK(f, cudaMemcpy(f->EyT, eyt.data(), eyt.size() * sizeof(float), cudaMemcpyHostToDevice));
     std::vector<float> s32((size_t)n);
     for (int y = 0; y < n; ++y) s32[(size_t)y] = (float)std::sin(kTwoPi * (double)(32l * y % n) / n);
     if ((r = falloc(f, &f->sin32, s32.size()))) return r;
@@ -171,7 +178,7 @@ int ensure_workspace(spgpe_fno *f, int B, int n) {
   const int splits = (int)std::max<size_t>(1, P / 1024);
   size_t wmax = std::max<size_t>((size_t)f->W * f->cin, (size_t)f->W * f->W);
   wmax = std::max(wmax, std::max((size_t)f->H * f->W, (size_t)f->cout * f->H));
-  f->part_n = (size_t)B * splits * wmax;
+  f->part_n = std::max((size_t)B * splits * wmax, (size_t)f->sms * (size_t)project_partials(f->H, f->cout));
   if ((r = falloc(f, &f->X1, rows * 2)) || (r = falloc(f, &f->hp, hid)) || (r = falloc(f, &f->h, hid)) ||
       (r = falloc(f, &f->dh, hid)) || (r = falloc(f, &f->dv, act)) || (r = falloc(f, &f->dv2, act)) ||
       (r = falloc(f, &f->dout, (size_t)B * f->cout * P)) || (r = falloc(f, &f->oh, spec)) ||
@@ -283,13 +290,17 @@ bool fused_mix(const spgpe_fno *f, int B) { return mix_applies(f->W, f->M) && B 
 
 bool use_layer(const spgpe_fno *f, int n) { return use_dft(f, n) && layer_applies(n, f->M, f->W); }
 
+bool use_head(const spgpe_fno *f, long P) {
+  return f->tensor_cores && f->sms > 0 && head_applies(f->W, f->H, f->cout, P);
+}
+
 // The kept modes of v [B][W][n][n] along x (with Exr, or Exi^T for the adjoint
 // of the inverse) and y: vh [B][W][2M][M].
 int spectrum(spgpe_fno *f, const float *v, bool adjoint, int B, int n, float2 *vh) {
   const long W = f->W, M = f->M, SP = 2 * M * M;
   if (use_dft(f, n)) {
-    FCK(f, dft_x(v, f->tab[(int)DftTable::X], adjoint, f->X1, (int)(B * W), n, f->M, f->sms, f->d_flags, f->st));
-    FCK(f, dft_y(f->X1, f->tab[(int)DftTable::Y], vh, (int)(B * W), n, f->M, f->sms, f->d_flags, f->st));
+    FCK(f, dft_x(v, f->Exr, adjoint, f->X1, (int)(B * W), n, f->M, f->st));
+    FCK(f, dft_y(f->X1, f->EyT, vh, (int)(B * W), n, f->M, f->st));
     return SPGPE_OK;
   }
   // X1 = v Exr, computed as X1^T = Exr^T v^T (the long side as N)
@@ -324,12 +335,17 @@ int forward(spgpe_fno *f, const float *a, int B, int n, float *out, bool keep) {
   const long WP = W * P;
   cudaStream_t st = f->st;
   // lift: v0 = P a + p
-  GemmR g = rg(W, P, f->cin, bfp(f, f->oP), true, f->cin, 1, a, P, 1, f->vs[0], P, 1);
-  g.batch = B;
-  g.sBb = (long)f->cin * P;
-  g.sCb = WP;
-  g.bias = f->wr + f->op;
-  FCK(f, greal(f, g, st));
+  GemmR g;
+  if (lift_applies(a, f->W, f->cin, P)) {
+    FCK(f, lift_forward(a, f->wr + f->oP, f->wr + f->op, f->vs[0], B, f->W, f->cin, P, st));
+  } else {
+    g = rg(W, P, f->cin, bfp(f, f->oP), true, f->cin, 1, a, P, 1, f->vs[0], P, 1);
+    g.batch = B;
+    g.sBb = (long)f->cin * P;
+    g.sCb = WP;
+    g.bias = f->wr + f->op;
+    FCK(f, greal(f, g, st));
+  }
   for (int l = 0; l < f->L; ++l) {
     float *v = f->vs[l], *u = f->us[l];
     if ((r = spectrum(f, v, false, B, n, f->vh[l]))) return r;
@@ -360,6 +376,11 @@ int forward(spgpe_fno *f, const float *a, int B, int n, float *out, bool keep) {
     }
   }
   // projection
+  if (use_head(f, P)) {
+    FCK(f, project_forward(f->vs[f->L], bfp(f, f->oQ1), f->wr + f->oq1, f->wr + f->oQ2, f->wr + f->oq2,
+                           keep ? f->hp : nullptr, out, B, f->W, f->cout, P, f->sms, f->d_flags, st));
+    return SPGPE_OK;
+  }
   g = rg(H, P, W, bfp(f, f->oQ1), true, W, 1, f->vs[f->L], P, 1, f->hp, P, 1);
   g.batch = B;
   g.sBb = WP;
@@ -388,21 +409,33 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
   cudaStream_t st = f->st;
   FCK(f, loss_terms(out, target, C * P, B, f->sums, f->dout, st));
   // output layer
-  if ((r = wgrad(f, C, H, P, B, f->dout, C * P, f->h, P, H * P, f->g + f->oQ2))) return r;
-  FCK(f, bias_gradient(f->dout, B, C, P, f->g + f->oq2, f->bscr, st));
-  GemmR g = rg(H, P, C, bfp(f, f->oQ2), true, 1, H, f->dout, P, 1, f->dh, P, 1);
-  g.batch = B;
-  g.sBb = C * P;
-  g.sCb = H * P;
-  FCK(f, greal(f, g, st));
-  FCK(f, gelu_backward(f->hp, f->dh, (long)B * H * P, st));
-  if ((r = wgrad(f, H, W, P, B, f->dh, H * P, f->vs[f->L], P, WP, f->g + f->oQ1))) return r;
-  FCK(f, bias_gradient(f->dh, B, H, P, f->g + f->oq1, f->bscr, st));
-  g = rg(W, P, H, bfp(f, f->oQ1), true, 1, W, f->dh, P, 1, f->dv, P, 1);
-  g.batch = B;
-  g.sBb = H * P;
-  g.sCb = WP;
-  FCK(f, greal(f, g, st));
+  GemmR g;
+  if (use_head(f, P)) {
+    int parts = 0;
+    FCK(f, project_gradient(f->dout, f->hp, f->wr + f->oQ2, f->dh, f->part, B, f->H, f->cout, P, f->sms, &parts, st));
+    const long np = project_partials(f->H, f->cout);
+    FCK(f, sum_parts(f->part, np, parts, C * H, f->g + f->oQ2, st));
+    FCK(f, sum_parts(f->part + C * H, np, parts, H, f->g + f->oq1, st));
+    FCK(f, sum_parts(f->part + C * H + H, np, parts, C, f->g + f->oq2, st));
+    if ((r = wgrad(f, H, W, P, B, f->dh, H * P, f->vs[f->L], P, WP, f->g + f->oQ1))) return r;
+    FCK(f, project_transpose(f->dh, bfp(f, f->oQ1), f->dv, B, f->W, P, f->sms, f->d_flags, st));
+  } else {
+    if ((r = wgrad(f, C, H, P, B, f->dout, C * P, f->h, P, H * P, f->g + f->oQ2))) return r;
+    FCK(f, bias_gradient(f->dout, B, C, P, f->g + f->oq2, f->bscr, st));
+    g = rg(H, P, C, bfp(f, f->oQ2), true, 1, H, f->dout, P, 1, f->dh, P, 1);
+    g.batch = B;
+    g.sBb = C * P;
+    g.sCb = H * P;
+    FCK(f, greal(f, g, st));
+    FCK(f, gelu_backward(f->hp, f->dh, (long)B * H * P, st));
+    if ((r = wgrad(f, H, W, P, B, f->dh, H * P, f->vs[f->L], P, WP, f->g + f->oQ1))) return r;
+    FCK(f, bias_gradient(f->dh, B, H, P, f->g + f->oq1, f->bscr, st));
+    g = rg(W, P, H, bfp(f, f->oQ1), true, 1, W, f->dh, P, 1, f->dv, P, 1);
+    g.batch = B;
+    g.sBb = H * P;
+    g.sCb = WP;
+    FCK(f, greal(f, g, st));
+  }
   float *du = f->dv, *dvn = f->dv2;
   for (int l = f->L - 1; l >= 0; --l) {
     // (the fused layer pass has multiplied du by the activation's derivative)

@@ -1,36 +1,25 @@
-// Truncated Fourier transforms of the neural operator's spectral layers on the
-// tensor cores (tcgen05): along x, X1[row][q] = sum_x v[row][x] T[x][q] (q =
-// 2 kx + part, real input); along y, vh[img][j][kx] = sum_y Ey[j][y] X1[img][y]
-// [kx]; and the inverse along y, G[img][y][kx] = sum_j conj(Ey[j][y])
-// oh[img][j][kx].
+// Truncated Fourier transforms of the neural operator's spectral layers: along
+// x, X1[row][q] = sum_x v[row][x] E[x][q] (q = 2 kx + part, real input); along
+// y, vh[img][j][kx] = sum_y Ey[j][y] X1[img][y][kx]; and the inverse along y,
+// G[img][y][kx] = sum_j conj(Ey[j][y]) oh[img][j][kx].
 //
-// Each is a product of a data operand (float32, from memory) with a constant
-// twiddle matrix, D[128 data rows][N columns] in tensor memory.  Both operands
-// are split into three bfloat16 terms, the first on a fixed grid (split3_grid:
-// the data scaled by a power of two per row, from the row's largest value),
-// so that the leading products add up exactly and the result keeps float32
-// accuracy: 16 flop per byte of data become 100, still below the tensor
-// cores' ratio, and the passes are bound by reading the data and by the
-// threads that split it.  The twiddle matrices are split on the host and
-// stored as the swizzled shared-memory image, fetched by bulk copies.
+// The forward transforms feed the spectral weights' gradients, where what is
+// left of a smooth field at high wavenumbers is as small as the transform's
+// own rounding; they are float32 sums in ascending order, one fma per term
+// (the order of the general products they replace, bit for bit), on the CUDA
+// cores, which 16 flop per byte keep busy: two packed fma per complex term or
+// pair of columns, operands from shared memory in wide reads, copied in
+// asynchronously one block ahead.
 //
-// Along y the kept wavenumbers are -M .. M - 1, so the complex product is taken
-// as cosine and sine sums of the data rows (img, kx, part): 2 (M + 1) columns
-// instead of the 4 M of the four real products, and lanes (kx, re), (kx, im)
-// of a warp combine them: vh(+-k) = C -+ i S.
+// The inverse along y runs on the tensor cores (tcgen05): D[128 data rows][N
+// columns] in tensor memory, data and twiddles split into three bfloat16
+// terms, the first on a fixed grid (split3_grid: the data scaled by a power of
+// two per row, from the row's largest value), so that the leading products add
+// up exactly and the result keeps float32 accuracy.  The kept wavenumbers are
+// -M .. M - 1, so the complex product is taken with cosines and sines of 0 .. M
+// only.  The twiddle matrix is split on the host and stored as the swizzled
+// shared-memory image, fetched by bulk copies.
 //
-// The transform kernel: 512 threads hold a whole unit of 128 rows x 256 k in
-// registers.  As a 64-wide block of it is split into one of two operand
-// buffers, the same registers take the block of the next unit, so that up to
-// 128 KB per SM are in flight; two sets of accumulators let a unit's results
-// leave while the next unit's first block is in the tensor cores.
-//
-// Measured on GB300 (256 images = batch 4 x 64 channels, 32 modes) against the
-// CUDA-core products they replace: at 256^2 along x 116 -> 32 us, along y 126
-// -> 13 us, inverse along y 76 -> 14 us; at 512^2 442 -> 208, 126 -> 23 and 129
-// -> 24 us.  With a plain three-term split (no grid) the accumulator's
-// truncation showed: the weights after eight training steps were 6.5e-6 off
-// the 64-bit result instead of 8e-7; with the grid they are 2 to 5e-7 off.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -49,240 +38,181 @@ namespace fno {
 
 namespace {
 
-constexpr int kThreads = 512;   // transforms
 constexpr int kThreadsI = 256;  // inverse along y
 constexpr size_t kTermA = (size_t)kTcRows * kRowBytes;  // one term of 128 rows x 64 k
 
-// columns of an accumulator: a multiple of 16
-__host__ __device__ constexpr int pad16(int v) { return (v + 15) / 16 * 16; }
+// 16 bytes global -> shared, asynchronous (both addresses 16-byte aligned).
+__device__ __forceinline__ void cp16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT> __device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
 
-struct DftArgs {
-  const float *src;
-  const unsigned char *tab;  // [n / 64 blocks][3 terms][N rows][128 bytes], swizzled
-  float *dst;
-  int n, M, ntiles;
-  float g0, g1;                // factors of the columns of kx = 0 and of the others (x transform)
-  int *flags;
-};
+// Along x: 128 rows x 8 CT columns per block (CT columns of 4 rows per thread),
+// blocks of 32 x.  A warp reads 4 x 4 rows and all columns: one shared-memory
+// wavefront per 16 bytes of a row, two per 4 columns, 20 for the 128 fma of 4 x.
+constexpr int kXRows = 128, kXBlock = 32, kXStride = kXBlock + 4;  // (rows shifted by 4 banks)
 
-template <int N, int NB> struct DftSmem {
-  static constexpr size_t kBlockB = (size_t)3 * N * kRowBytes;
-  static constexpr size_t kA = 2 * 3 * kTermA;
-  static constexpr size_t kBytes = 1024 + kA + NB * kBlockB + (2 * kTcRows + kThreads) * sizeof(float) + 64;
-};
-
-// ALONG_Y false: data rows are contiguous rows of n values (x transform);
-// true: data row r = img 2M + q holds X1[img][y][q], y = 0..n-1.  A unit is a
-// tile of 128 rows over a segment of NB blocks of 64 k: the whole row for grids
-// up to 256.  Larger rows take several segments, each with its own scales,
-// added up in memory by the thread that owns the value; a CTA runs all its
-// tiles through one segment, whose part of the table stays in shared memory,
-// before the next.
-template <int N, int NB, bool ALONG_Y>
-__global__ void __launch_bounds__(kThreads, 1) dft(const DftArgs a) {
-  using S = DftSmem<N, NB>;
-  constexpr uint32_t kCols = 512;  // two units' accumulators, 3 N columns from 0 and from 256
-  static_assert(3 * N <= 256, "three accumulators within half of the tensor memory");
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char *sm =
-      reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int nseg = a.n / (NB * kKBlock);
-  unsigned char *sB = sm + S::kA;
-  float *rowmax = reinterpret_cast<float *>(sB + NB * S::kBlockB);        // [unit parity][row] largest value
-  float *quarter = rowmax + 2 * kTcRows;                                  // [thread] maxima of quarter rows (along y)
-  uint64_t *mma = reinterpret_cast<uint64_t *>(quarter + kThreads);       // [2] operand buffer's MMAs done
-  uint64_t *full = mma + 2;                                               // the segment's table landed
-  uint32_t *slot = reinterpret_cast<uint32_t *>(full + 1);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int q2 = 2 * a.M;
-  const int mytiles = (a.ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int units = mytiles * nseg;
-  auto tile_of = [&](int u) { return (int)blockIdx.x + (u % mytiles) * (int)gridDim.x; };
-
-  auto fetch_b = [&](int seg) {  // thread 0: a segment's part of the table
-    mbar_expect_tx(full, (uint32_t)(NB * S::kBlockB));
-    for (int k = 0; k < NB; ++k)
-      bulk_g2s(sB + k * S::kBlockB, a.tab + (size_t)(seg * NB + k) * S::kBlockB, (uint32_t)S::kBlockB, full);
-  };
-  if (warp == 0) {
-    tmem_alloc(slot, kCols);
-    tmem_relinquish();
-  }
-  if (tid == 0) {
-    for (int i = 0; i < 2; ++i) mbar_init(&mma[i], 1);
-    mbar_init(full, 1);
-    mbar_fence_init();
-    fetch_b(0);
-  }
-
-  // The thread's part of a block: two runs of 8 k.  Along x: rows (tid >> 3) +
-  // 64 i, run tid & 7, in the order of x_slot (4 of the block's first 32 k and 4
-  // of the others, so that 8 lanes read whole 128-byte lines); along y: row tid & 127, runs (tid >> 7) + 4 i.
-  float x[NB][16], c[2];
-  auto load = [&](int u, int kc) {
-    const int tile = tile_of(u), kb = (u / mytiles) * NB + kc;
-    if constexpr (!ALONG_Y) {
+template <int CT>
+__global__ void __launch_bounds__(256, 2) dft_rows(const float *__restrict__ v, const float *__restrict__ E, int n, int q2,
+                                                   float g0, float g1, float *__restrict__ out) {
+  constexpr int N = 8 * CT, P = CT / 2;  // columns (padded), packed pairs per thread
+  extern __shared__ __align__(16) float smem_f[];
+  float *sv = smem_f, *se = smem_f + 2 * kXRows * kXStride;  // [2][row][kXStride], [2][x][N]
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const long row0 = (long)blockIdx.x * kXRows;
+  const int blocks = n / kXBlock;
+  auto fetch = [&](int b) {
+    float *dv = sv + (b & 1) * kXRows * kXStride, *de = se + (b & 1) * kXBlock * N;
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const float4 *p = reinterpret_cast<const float4 *>(
-            a.src + (long)(tile * kTcRows + (tid >> 3) + 64 * i) * a.n + kb * kKBlock + (tid & 7) * 4);
-        const float4 v = p[0], w = p[8];
-        x[kc][8 * i] = v.x; x[kc][8 * i + 1] = v.y; x[kc][8 * i + 2] = v.z; x[kc][8 * i + 3] = v.w;
-        x[kc][8 * i + 4] = w.x; x[kc][8 * i + 5] = w.y; x[kc][8 * i + 6] = w.z; x[kc][8 * i + 7] = w.w;
-      }
-    } else {
-      const int r = tile * kTcRows + (tid & 127), img = r / q2, q = r - img * q2;
-      const float *p = a.src + ((long)img * a.n + kb * kKBlock) * q2 + q;
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) x[kc][8 * i + j] = p[(long)(((tid >> 7) + 4 * i) * 8 + j) * q2];
+    for (int i = 0; i < kXRows * kXBlock / 4 / 256; ++i) {
+      const int e = tid + 256 * i, r = e >> 3, c = e & 7;
+      cp16(dv + r * kXStride + 4 * c, v + (row0 + r) * n + b * kXBlock + 4 * c);
     }
-  };
-  // the scales of the unit in x, from its rows' largest magnitudes
-  auto scale = [&](int parity) {
-    float vm[2] = {0.f, 0.f};
-#pragma unroll
-    for (int k = 0; k < NB; ++k)
-#pragma unroll
-      for (int j = 0; j < 16; ++j) vm[ALONG_Y ? 0 : j / 8] = fmaxf(vm[ALONG_Y ? 0 : j / 8], fabsf(x[k][j]));
-    if constexpr (!ALONG_Y) {  // 8 lanes hold a row
-      __syncthreads();         // the unit that had this slot of rowmax is out
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) vm[i] = fmaxf(vm[i], __shfl_xor_sync(0xffffffffu, vm[i], o));
-        c[i] = grid_scale(vm[i]);
-        if ((tid & 7) == 0) rowmax[parity * kTcRows + (tid >> 3) + 64 * i] = vm[i];
-      }
-    } else {  // four threads hold a row
-      quarter[tid] = vm[0];
-      __syncthreads();
-      const int r = tid & 127;
-      const float v = fmaxf(fmaxf(quarter[r], quarter[r + 128]), fmaxf(quarter[r + 256], quarter[r + 384]));
-      c[0] = c[1] = grid_scale(v);
-      if (tid < 128) rowmax[parity * kTcRows + tid] = v;
+    for (int e = tid; e < kXBlock * q2 / 4; e += 256) {
+      const int x = 4 * e / q2, c = 4 * e - x * q2;
+      cp16(de + x * N + c, E + (long)(b * kXBlock + x) * q2 + c);
     }
+    cp_commit();
   };
-  auto store = [&](unsigned char *sA, int kc) {
+  for (int e = tid; e < 2 * kXBlock * N; e += 256)
+    if (e % N >= q2) se[e] = 0.f;  // the columns of the padding
+  float2 acc[4][P];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int row = ALONG_Y ? (tid & 127) : (tid >> 3) + 64 * i, ch = ALONG_Y ? (tid >> 7) + 4 * i : (tid & 7);
-      const float v[8] = {x[kc][8 * i],     x[kc][8 * i + 1], x[kc][8 * i + 2], x[kc][8 * i + 3],
-                          x[kc][8 * i + 4], x[kc][8 * i + 5], x[kc][8 * i + 6], x[kc][8 * i + 7]};
-      uint4 h, m, l;
-      split3_grid(v, c[i], h, m, l);
-      const uint32_t off = sw128(row, ch);
-      *reinterpret_cast<uint4 *>(sA + off) = h;
-      *reinterpret_cast<uint4 *>(sA + kTermA + off) = m;
-      *reinterpret_cast<uint4 *>(sA + 2 * kTermA + off) = l;
-    }
-  };
-  for (int k = 0; k < NB; ++k) load(0, k);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *slot;
-  // results of a unit: lane 32 (warp & 3) + lane of the accumulators is the
-  // data row; the four groups of four warps take alternate groups of 8 columns
-  auto epilogue = [&](int u) {
-    const int lr = 32 * (warp & 3) + lane, r = tile_of(u) * kTcRows + lr;
-    const bool more = u >= mytiles;  // add to the segments before
-    const uint32_t base = tmem + 256 * (u & 1) + ((uint32_t)(32 * (warp & 3)) << 16);
-    const float un = grid_unscale(rowmax[(u & 1) * kTcRows + lr]);
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < P; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  fetch(0);
 #pragma unroll 1
-    for (int g = warp >> 2; g < N / 8; g += 4) {
-      float v[8], w[8], z[8];
-      tmem_ld8(base + 8 * g, v);
-      tmem_ld8(base + N + 8 * g, w);
-      tmem_ld8(base + 2 * N + 8 * g, z);
-      tmem_ld_wait();
+  for (int b = 0; b < blocks; ++b) {
+    if (b + 1 < blocks) {
+      fetch(b + 1);
+      cp_wait<1>();
+    } else {
+      cp_wait<0>();
+    }
+    __syncthreads();
+    const float *pv = sv + (b & 1) * kXRows * kXStride + 4 * ty * kXStride, *pe = se + (b & 1) * kXBlock * N + CT * tx;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = (v[i] + (w[i] + z[i])) * un;
-      if constexpr (!ALONG_Y) {
-        float *o = a.dst + (long)r * q2 + 8 * g;
+    for (int k = 0; k < kXBlock; k += 4) {
+      float a[4][4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] *= g == 0 && i < 2 ? a.g0 : a.g1;
+      for (int i = 0; i < 4; ++i) {
+        const float4 t = *reinterpret_cast<const float4 *>(pv + i * kXStride + k);
+        a[i][0] = t.x; a[i][1] = t.y; a[i][2] = t.z; a[i][3] = t.w;
+      }
 #pragma unroll
-        for (int i = 0; i < 8; i += 4)
-          if (8 * g + i < q2) {
-            float4 s = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            if (more) {
-              const float4 p = *reinterpret_cast<const float4 *>(o + i);
-              s = make_float4(p.x + s.x, p.y + s.y, p.z + s.z, p.w + s.w);
-            }
-            *reinterpret_cast<float4 *>(o + i) = s;
+      for (int kk = 0; kk < 4; ++kk) {
+        float2 w[P];
+        if constexpr (CT % 4 == 0) {
+#pragma unroll
+          for (int j = 0; j < P; j += 2) {
+            const float4 t = *reinterpret_cast<const float4 *>(pe + (k + kk) * N + 2 * j);
+            w[j] = make_float2(t.x, t.y);
+            w[j + 1] = make_float2(t.z, t.w);
           }
-      } else {
-        const int img = r / q2, q = r - img * q2;
-        float *o = a.dst + (long)img * q2 * q2 + q;
+        } else {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int k = 4 * g + i;  // columns 2k, 2k + 1: cosine and sine sums of wavenumber k
-          const float sp = __shfl_xor_sync(0xffffffffu, v[2 * i + 1], 1);
-          const float s = (q & 1) ? -sp : sp;
-          if (k < a.M) {
-            float *e = o + (long)k * q2;
-            *e = more ? *e + (v[2 * i] + s) : v[2 * i] + s;
-          }
-          if (k >= 1 && k <= a.M) {
-            float *e = o + (long)(q2 - k) * q2;
-            *e = more ? *e + (v[2 * i] - s) : v[2 * i] - s;
-          }
+          for (int j = 0; j < P; ++j) w[j] = *reinterpret_cast<const float2 *>(pe + (k + kk) * N + 2 * j);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < P; ++j) acc[i][j] = __ffma2_rn(w[j], make_float2(a[i][kk], a[i][kk]), acc[i][j]);
+      }
+    }
+    __syncthreads();  // the block's buffers are read: the block after next may go there
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float *o = out + (row0 + 4 * ty + i) * q2 + CT * tx;
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+      const float g = CT * tx + 2 * j == 0 ? g0 : g1;
+      if (CT * tx + 2 * j < q2) *reinterpret_cast<float2 *>(o + 2 * j) = make_float2(acc[i][j].x * g, acc[i][j].y * g);
+    }
+  }
+}
+
+// Along y: one image per 128 threads (or several small ones), 4 wavenumbers j x
+// 4 kx per thread, blocks of 32 y.  The complex term a b is two packed fma:
+// (-a.y, a.y) (b.y, b.x), then (a.x, a.x) (b.x, b.y).
+constexpr int kYBlock = 32;
+
+__global__ void __launch_bounds__(128) dft_cols(const float2 *__restrict__ X1, const float2 *__restrict__ Et, int n,
+                                                int M, int images, int per_block, float2 *__restrict__ out) {
+  extern __shared__ __align__(16) float2 smem_c[];
+  const int J = 2 * M, jt = (J + 3) / 4, kt = (M + 3) / 4, Jp = 4 * jt, Kp = 4 * kt;  // padded to whole thread tiles
+  float2 *se = smem_c, *sx = smem_c + 2 * kYBlock * Jp;  // [2][y][Jp], [2][image][y][Kp]
+  const int tid = threadIdx.x, per = jt * kt;
+  const int im = min(tid / per, per_block - 1), loc = tid % per, tj = loc / kt, tk = loc - tj * kt;
+  const int img0 = blockIdx.x * per_block;
+  const bool mine = tid < per * per_block && img0 + im < images;
+  const int blocks = n / kYBlock;
+  for (int e = tid; e < 2 * kYBlock * Jp; e += 128)
+    if (e % Jp >= J) se[e] = make_float2(0.f, 0.f);
+  for (int e = tid; e < 2 * per_block * kYBlock * Kp; e += 128)
+    if (e % Kp >= M) sx[e] = make_float2(0.f, 0.f);
+  auto fetch = [&](int b) {
+    float2 *de = se + (b & 1) * kYBlock * Jp, *dx = sx + (b & 1) * per_block * kYBlock * Kp;
+    for (int e = tid; e < kYBlock * M; e += 128) {  // two wavenumbers at a time (2M of them per y)
+      const int y = e / M, c = 2 * (e - y * M);
+      cp16(de + y * Jp + c, Et + (long)(b * kYBlock + y) * J + c);
+    }
+    const int h = M / 2;  // pairs of kx per y (M is even)
+    for (int e = tid; e < per_block * kYBlock * h; e += 128) {
+      const int i = e / (kYBlock * h), r = e - i * kYBlock * h, y = r / h, c = 2 * (r - y * h);
+      if (img0 + i < images) cp16(dx + (i * kYBlock + y) * Kp + c, X1 + ((long)(img0 + i) * n + b * kYBlock + y) * M + c);
+    }
+    cp_commit();
+  };
+  float2 acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  fetch(0);
+#pragma unroll 1
+  for (int b = 0; b < blocks; ++b) {
+    if (b + 1 < blocks) {
+      fetch(b + 1);
+      cp_wait<1>();
+    } else {
+      cp_wait<0>();
+    }
+    __syncthreads();
+    const float2 *pe = se + (b & 1) * kYBlock * Jp + 4 * tj;
+    const float2 *px = sx + ((b & 1) * per_block + im) * kYBlock * Kp + 4 * tk;
+#pragma unroll 4
+    for (int y = 0; y < kYBlock; ++y) {
+      const float4 e0 = *reinterpret_cast<const float4 *>(pe + y * Jp), e1 = *reinterpret_cast<const float4 *>(pe + y * Jp + 2);
+      const float4 x0 = *reinterpret_cast<const float4 *>(px + y * Kp), x1 = *reinterpret_cast<const float4 *>(px + y * Kp + 2);
+      const float2 a[4] = {{e0.x, e0.y}, {e0.z, e0.w}, {e1.x, e1.y}, {e1.z, e1.w}};
+      const float2 x[4] = {{x0.x, x0.y}, {x0.z, x0.w}, {x1.x, x1.y}, {x1.z, x1.w}};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float2 s = make_float2(x[k].y, x[k].x);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          acc[j][k] = __ffma2_rn(make_float2(-a[j].y, a[j].y), s, acc[j][k]);
+          acc[j][k] = __ffma2_rn(make_float2(a[j].x, a[j].x), x[k], acc[j][k]);
         }
       }
     }
-    tc_fence_before();
-  };
-
-  bool ok = true;
-  int g = 0;  // block counter: operand buffer g & 1, its MMAs' phase (g >> 1) & 1
-#pragma unroll 1
-  for (int u = 0; u < units && ok; ++u) {
-    scale(u & 1);
-    const int seg = u / mytiles;
-    if (u > 0 && u % mytiles == 0) {  // the next segment's table, once nothing reads the one before
-      ok = mbar_wait_bounded(&mma[(g - 1) & 1], (uint32_t)(((g - 1) >> 1) & 1));
-      if (tid == 0 && ok) fetch_b(seg);
-    }
+    __syncthreads();  // the block's buffers are read: the block after next may go there
+  }
+  if (!mine) return;
+  float2 *o = out + (long)(img0 + im) * J * M;
 #pragma unroll
-    for (int kc = 0; kc < NB; ++kc, ++g) {
-      const int s = g & 1;
-      if (g >= 2) ok = mbar_wait_bounded(&mma[s], (uint32_t)(((g >> 1) - 1) & 1)) && ok;
-      unsigned char *sA = sm + s * 3 * kTermA;
-      store(sA, kc);
-      if (u + 1 < units) load(u + 1, kc);
-      fence_proxy_async();
-      ok = __syncthreads_and(ok);
-      if (tid == 0) {
-        // (the commit follows in any case, so that every wait ends)
-        const bool landed = mbar_wait_bounded(full, (uint32_t)(seg & 1));
-        if (!landed || !ok) atomicOr(a.flags, kErrTimeout);
-        if (!landed) mbar_wait_bounded(full, (uint32_t)(seg & 1));  // the copy may still land: once more before the buffer can go
-        tc_fence_after();
-        if (landed && ok)
-          umma_split33<N>(tmem + 256 * (u & 1), sA, kTermA, sB + kc * S::kBlockB, kc > 0);
-        umma_commit(&mma[s]);
-      }
-      // the unit before leaves while this unit's first block is in the tensor cores
-      if (kc == 0 && u > 0) {
-        ok = mbar_wait_bounded(&mma[s ^ 1], (uint32_t)(((g - 1) >> 1) & 1)) && ok;
-        tc_fence_after();
-        if (ok) epilogue(u - 1);
-      }
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int k = 0; k < 4; k += 2) {
+      const int jj = 4 * tj + j, kk = 4 * tk + k;  // (M is even: kk < M holds for the pair)
+      if (jj < J && kk < M)
+        *reinterpret_cast<float4 *>(o + (long)jj * M + kk) = make_float4(acc[j][k].x, acc[j][k].y, acc[j][k + 1].x, acc[j][k + 1].y);
     }
-  }
-  // everything issued is complete before the buffers go; then the last unit
-  ok = mbar_wait_bounded(&mma[(g - 1) & 1], (uint32_t)(((g - 1) >> 1) & 1)) && ok;
-  tc_fence_after();
-  if (ok) epilogue(units - 1);
-  else if (tid == 0) atomicOr(a.flags, kErrTimeout);
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
-    tc_fence_after();
-    tmem_dealloc(tmem, kCols);
-  }
 }
 
 // Inverse along y: data row r = img 2M + q of 128 and a tile of NY rows y per
@@ -443,21 +373,16 @@ template <class K> cudaError_t grant(K kern, size_t smem, size_t &granted) {
   return cudaSuccess;
 }
 
-template <int N, int NB, bool ALONG_Y> cudaError_t launch_dft_nb(DftArgs a, int sms, cudaStream_t st) {
-  auto kern = dft<N, NB, ALONG_Y>;
-  constexpr size_t smem = DftSmem<N, NB>::kBytes;
-  static_assert(smem <= 227 * 1024, "operand buffers and a segment of the table within a block's limit");
+template <int CT>
+cudaError_t launch_rows(const float *v, const float *E, int n, int q2, float g0, float g1, float *out, long rows,
+                        cudaStream_t st) {
+  auto kern = dft_rows<CT>;
+  constexpr size_t smem = (size_t)2 * (kXRows * kXStride + kXBlock * 8 * CT) * sizeof(float);
   static size_t granted = 0;
   const cudaError_t e = grant(kern, smem, granted);
   if (e != cudaSuccess) return e;
-  kern<<<std::max(1, std::min(a.ntiles, sms)), kThreads, smem, st>>>(a);
+  kern<<<(unsigned)(rows / kXRows), 256, smem, st>>>(v, E, n, q2, g0, g1, out);
   return cudaGetLastError();
-}
-
-template <int N, bool ALONG_Y> cudaError_t launch_dft(const DftArgs &a, int sms, cudaStream_t st) {
-  if (a.n == 64) return launch_dft_nb<N, 1, ALONG_Y>(a, sms, st);
-  if (a.n == 128) return launch_dft_nb<N, 2, ALONG_Y>(a, sms, st);
-  return launch_dft_nb<N, 4, ALONG_Y>(a, sms, st);
 }
 
 template <int NY> cudaError_t launch_idft(const IdftArgs &a, int rows, cudaStream_t st) {
@@ -501,38 +426,7 @@ bool dft_applies(int n, int modes, int width) {
 
 // (The twiddles are the float32 ones of the general path, so that both paths
 // compute the same transform.)
-// Slot of x in its 64-wide block: run r = slot / 8 holds x = 4 r .. 4 r + 3 and
-// 32 + 4 r .. 32 + 4 r + 3.
-static int x_slot(int x) {
-  const int k = x % kKBlock;
-  return 8 * ((k % 32) / 4) + k % 4 + (k >= 32 ? 4 : 0);
-}
-
 std::vector<uint16_t> dft_table(DftTable which, int n, int M) {
-  if (which == DftTable::X) {  // columns 2k, 2k + 1 = cos, -sin(2 pi k x / n), k < M
-    const int N = pad16(2 * M);
-    std::vector<uint16_t> t((size_t)(n / kKBlock) * 3 * N * kKBlock, 0);
-    for (int x = 0; x < n; ++x)
-      for (int k = 0; k < M; ++k) {
-        const double th = kTwoPi * (double)((long)k * x % n) / n;
-        uint16_t *b = t.data() + (size_t)(x / kKBlock) * 3 * N * kKBlock;
-        put3(b, N, 2 * k, x_slot(x), (float)std::cos(th));
-        put3(b, N, 2 * k + 1, x_slot(x), (float)-std::sin(th));
-      }
-    return t;
-  }
-  if (which == DftTable::Y) {  // columns 2k, 2k + 1 = cos, sin(2 pi k y / n), k = 0..M
-    const int N = pad16(2 * (M + 1));
-    std::vector<uint16_t> t((size_t)(n / kKBlock) * 3 * N * kKBlock, 0);
-    for (int y = 0; y < n; ++y)
-      for (int k = 0; k <= M; ++k) {
-        const double th = kTwoPi * (double)((long)k * y % n) / n;
-        uint16_t *b = t.data() + (size_t)(y / kKBlock) * 3 * N * kKBlock;
-        put3(b, N, 2 * k, y % kKBlock, (float)std::cos(th));
-        put3(b, N, 2 * k + 1, y % kKBlock, (float)std::sin(th));
-      }
-    return t;
-  }
   if (which == DftTable::LayerX) {  // row x, slots 2k, 2k + 1 = cos, -sin(2 pi k x / n), k < M; tiles of 128 rows
     std::vector<uint16_t> t((size_t)((n + kTcRows - 1) / kTcRows) * 3 * kTcRows * kKBlock, 0);
     for (int x = 0; x < n; ++x)
@@ -559,32 +453,28 @@ std::vector<uint16_t> dft_table(DftTable which, int n, int M) {
   return t;
 }
 
-cudaError_t dft_x(const float *v, const void *table, bool adjoint, float *X1, int images, int n, int modes, int sms,
-                  int *flags, cudaStream_t st) {
-  const float w = adjoint ? (float)(1.0 / ((double)n * n)) : 1.f;
-  const DftArgs a{v, static_cast<const unsigned char *>(table), X1, n, modes, (int)((long)images * n / kTcRows),
-                  w, adjoint ? 2.f * w : w, flags};
-  switch (pad16(2 * modes)) {
-    case 16: return launch_dft<16, false>(a, sms, st);
-    case 32: return launch_dft<32, false>(a, sms, st);
-    case 48: return launch_dft<48, false>(a, sms, st);
-    case 64: return launch_dft<64, false>(a, sms, st);
+cudaError_t dft_x(const float *v, const float *E, bool adjoint, float *X1, int images, int n, int modes, cudaStream_t st) {
+  const float w = adjoint ? (float)(1.0 / ((double)n * n)) : 1.f, g1 = adjoint ? 2.f * w : w;  // powers of two: exact
+  const long rows = (long)images * n;
+  const int q2 = 2 * modes;
+  switch ((q2 + 15) / 16) {
+    case 1: return launch_rows<2>(v, E, n, q2, w, g1, X1, rows, st);
+    case 2: return launch_rows<4>(v, E, n, q2, w, g1, X1, rows, st);
+    case 3: return launch_rows<6>(v, E, n, q2, w, g1, X1, rows, st);
+    case 4: return launch_rows<8>(v, E, n, q2, w, g1, X1, rows, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t dft_y(const float *X1, const void *table, float2 *vh, int images, int n, int modes, int sms, int *flags,
-                  cudaStream_t st) {
-  const DftArgs a{X1, static_cast<const unsigned char *>(table), reinterpret_cast<float *>(vh), n, modes,
-                  (int)((long)images * 2 * modes / kTcRows), 1.f, 1.f, flags};
-  switch (pad16(2 * (modes + 1))) {
-    case 16: return launch_dft<16, true>(a, sms, st);
-    case 32: return launch_dft<32, true>(a, sms, st);
-    case 48: return launch_dft<48, true>(a, sms, st);
-    case 64: return launch_dft<64, true>(a, sms, st);
-    case 80: return launch_dft<80, true>(a, sms, st);
-    default: return cudaErrorInvalidValue;
-  }
+cudaError_t dft_y(const float *X1, const float2 *Et, float2 *vh, int images, int n, int modes, cudaStream_t st) {
+  const int jt = (2 * modes + 3) / 4, kt = (modes + 3) / 4, per_block = std::max(1, 128 / (jt * kt));
+  const size_t smem = (size_t)2 * kYBlock * (4 * jt + per_block * 4 * kt) * sizeof(float2);
+  static size_t granted = 48 * 1024;
+  const cudaError_t e = grant(dft_cols, smem, granted);
+  if (e != cudaSuccess) return e;
+  dft_cols<<<(unsigned)((images + per_block - 1) / per_block), 128, smem, st>>>(reinterpret_cast<const float2 *>(X1), Et, n,
+                                                                               modes, images, per_block, vh);
+  return cudaGetLastError();
 }
 
 cudaError_t idft_y(const float2 *oh, const void *table, const float *sin32, float2 *G, int images, int n, int modes,

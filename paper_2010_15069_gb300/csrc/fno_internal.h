@@ -57,20 +57,18 @@ bool gemm_tc_applies(const GemmR &g);
 cudaError_t gemm_real_tc(const GemmR &g, cudaStream_t st);
 cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool accumulate, cudaStream_t st);
 cudaError_t gemm_complex(const GemmC &g, cudaStream_t st);
-// Truncated Fourier transforms on the tensor cores (fno_dft.cu) of `images` n x n
-// fields with the kept modes kx < M, ky = -M .. M - 1 (M even, at most 32; n a
-// multiple of 64; `width` channels per sample, whose rows fill whole tiles of 128):
-// along x (cos, -sin; adjoint: times g_k / n^2, g_0 = 1, g_k = 2), along y, and
-// the inverse along y.
-// Tables: dft_table on the host, uploaded as they are; sin32[y] = sin(2 pi 32
-// y / n).  flags receives a wait that ran out.
-enum class DftTable { X, Y, InverseY, LayerX };
+// Truncated Fourier transforms (fno_dft.cu) of `images` n x n fields with the
+// kept modes kx < M, ky = -M .. M - 1 (M even, at most 32; n a multiple of 64;
+// `width` channels per sample, whose rows fill whole tiles of 128): along x
+// (E[x][2 k + part] = cos, -sin; adjoint: times g_k / n^2, g_0 = 1, g_k = 2) and
+// along y (Et[y][j] = exp(-2 pi i ky_j y / n)) in float32, the inverse along y
+// on the tensor cores (table: dft_table(InverseY) as it is; sin32[y] = sin(2 pi
+// 32 y / n)); flags receives a wait that ran out.
+enum class DftTable { InverseY, LayerX };
 bool dft_applies(int n, int modes, int width);
 std::vector<uint16_t> dft_table(DftTable which, int n, int modes);
-cudaError_t dft_x(const float *v, const void *table, bool adjoint, float *X1, int images, int n, int modes, int sms,
-                  int *flags, cudaStream_t st);
-cudaError_t dft_y(const float *X1, const void *table, float2 *vh, int images, int n, int modes, int sms, int *flags,
-                  cudaStream_t st);
+cudaError_t dft_x(const float *v, const float *E, bool adjoint, float *X1, int images, int n, int modes, cudaStream_t st);
+cudaError_t dft_y(const float *X1, const float2 *Et, float2 *vh, int images, int n, int modes, cudaStream_t st);
 cudaError_t idft_y(const float2 *oh, const void *table, const float *sin32, float2 *G, int images, int n, int modes,
                    int *flags, cudaStream_t st);
 // The rest of a spectral layer in one pass (fno_layer.cu; W = 32 or 64 where
@@ -84,6 +82,27 @@ cudaError_t layer_forward(const float *v, const float2 *G, const void *table, co
                           int *flags, cudaStream_t st);
 cudaError_t layer_backward(const float *du, const float2 *G, const void *table, const void *weights, const float *u_prev,
                            float *out, int batch, int width, int n, int modes, int sms, int *flags, cudaStream_t st);
+// Lift and projection (fno_head.cu).  head_applies: W = 32 or 64 channels, 2 W
+// hidden ones, at most 4 outputs, P a multiple of 128.  project_forward: out =
+// Q2 gelu(Q1 v + q1) + q2, Q1 v + q1 to hp unless null.  project_gradient: dhp =
+// (Q2^T dout) gelu'(hp) and, per CTA (*parts of them), the sums dQ2 [cout][H],
+// dq1 [H], dq2 [cout] in project_partials() floats.  project_transpose: dv =
+// Q1^T dhp.  lift_forward: v = A a + bias.
+bool head_applies(int width, int hidden, int cout, long P);
+cudaError_t project_forward(const float *v, const void *q1w, const float *q1b, const float *q2w, const float *q2b,
+                            float *hp, float *out, int batch, int width, int cout, long P, int sms, int *flags,
+                            cudaStream_t st);
+long project_partials(int hidden, int cout);
+cudaError_t project_gradient(const float *dout, const float *hp, const float *q2w, float *dhp, float *part, int batch,
+                             int hidden, int cout, long P, int sms, int *parts, cudaStream_t st);
+cudaError_t project_transpose(const float *dhp, const void *q1w, float *dv, int batch, int width, long P, int sms,
+                              int *flags, cudaStream_t st);
+bool lift_applies(const float *in, int width, int cin, long P);
+cudaError_t lift_forward(const float *in, const float *w, const float *bias, float *v, int batch, int width, int cin,
+                         long P, cudaStream_t st);
+// out[i] = sum of part[k][i] over k < parts, in a fixed order; stride floats
+// from one part to the next.
+cudaError_t sum_parts(const float *part, long stride, int parts, long n, float *out, cudaStream_t st);
 cudaError_t gelu_forward(const float *u, float *v, long n, cudaStream_t st);
 cudaError_t gelu_backward(const float *u, float *d, long n, cudaStream_t st);
 // grad[c] = sum over the batch and the points of x[b][c][p]; scratch holds
@@ -109,6 +128,12 @@ __device__ __forceinline__ void adam_one(float &w, float &m, float &v, float g, 
 __device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_d(float x) {
   return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
+}
+// Both of them (one erf).
+__device__ __forceinline__ void gelu_both(float x, float &g, float &d) {
+  const float phi = 0.5f * (1.f + erff(x * 0.70710678118654752f));
+  g = x * phi;
+  d = phi + x * expf(-0.5f * x * x) * 0.39894228040143268f;
 }
 // Up to kRanges [begin, end) ranges of the parameter vector.
 constexpr int kRanges = 16;

@@ -207,6 +207,25 @@ __global__ void reduce_splits(const float *__restrict__ part, long n, int splits
   }
 }
 
+// The same for few outputs and many parts: 8 threads per output, each every
+// eighth part, their sums added in order.
+__global__ void __launch_bounds__(256) sum_parts_k(const float *__restrict__ part, long stride, int parts, long n,
+                                                   float *out) {
+  __shared__ float red[8][33];
+  const int j = threadIdx.x & 31, s = threadIdx.x >> 5;
+  const long i = (long)blockIdx.x * 32 + j;
+  float v = 0.f;
+  if (i < n)
+    for (int k = s; k < parts; k += 8) v += part[(long)k * stride + i];
+  red[s][j] = v;
+  __syncthreads();
+  if (s == 0 && i < n) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) v += red[q][j];
+    out[i] = v;
+  }
+}
+
 struct c2 {
   float x, y;
 };
@@ -455,6 +474,11 @@ cudaError_t gemm_real(const GemmR &g, cudaStream_t st) {
 
 cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool accumulate, cudaStream_t st) {
   reduce_splits<<<grid_for(n), 256, 0, st>>>(part, n, splits, out, accumulate ? 1 : 0);
+  return cudaGetLastError();
+}
+
+cudaError_t sum_parts(const float *part, long stride, int parts, long n, float *out, cudaStream_t st) {
+  sum_parts_k<<<(unsigned)((n + 31) / 32), 256, 0, st>>>(part, stride, parts, n, out);
   return cudaGetLastError();
 }
 

@@ -218,24 +218,24 @@ __global__ void __launch_bounds__(kThreads, 1) layer(const LayerArgs a) {
     }
   };
 
-  bool ok = true;
+  bool ok = true, go = true;  // the thread's waits, and those of the whole block (what it leaves the loop by)
   float up[RUNS][8];
 #pragma unroll 1
-  for (int t = 0; t < tiles && ok; ++t) {
+  for (int t = 0; t < tiles && go; ++t) {
     const int s = t & 1;
     if (t > 0) load_u(t - 1, up);
-    if (t >= 2) ok = mbar_wait_bounded(&mma[s], (uint32_t)(((t >> 1) - 1) & 1));
+    if (t >= 2) ok = mbar_wait_bounded(&mma[s], (uint32_t)(((t >> 1) - 1) & 1)) && ok;
     store(s, t % 3);
     if (t + 1 < tiles) load(t + 1);
     fence_proxy_async();
-    ok = __syncthreads_and(ok);
+    go = __syncthreads_and(ok);
     if (tid == 0) {
       // (the commit follows in any case, so that every wait ends)
       const bool landed = t > 0 || mbar_wait_bounded(full, 0);
-      if (!landed || !ok) atomicOr(a.flags, kErrTimeout);
+      if (!landed || !go) atomicOr(a.flags, kErrTimeout);
       if (!landed) mbar_wait_bounded(full, 0);
       tc_fence_after();
-      if (landed && ok) {
+      if (landed && go) {
         const uint32_t d = tmem + 256 * s;
         const uint64_t wd = sw128_desc(sW);
 #pragma unroll 1
@@ -249,17 +249,18 @@ __global__ void __launch_bounds__(kThreads, 1) layer(const LayerArgs a) {
       umma_commit(&mma[s]);
     }
     if (t > 0) {
-      ok = mbar_wait_bounded(&mma[s ^ 1], (uint32_t)(((t - 1) >> 1) & 1)) && ok;
+      // (the tensor-memory loads need a warp's lanes together)
+      ok = __all_sync(0xffffffffu, mbar_wait_bounded(&mma[s ^ 1], (uint32_t)(((t - 1) >> 1) & 1)) && ok);
       tc_fence_after();
       if (ok) epilogue(t - 1, up);
     }
-    if (!ok || t + 1 == tiles) {
-      ok = mbar_wait_bounded(&mma[s], (uint32_t)((t >> 1) & 1)) && ok;
+    if (!go || t + 1 == tiles) {
+      ok = __all_sync(0xffffffffu, mbar_wait_bounded(&mma[s], (uint32_t)((t >> 1) & 1)) && ok);
       tc_fence_after();
-      if (ok) {
+      if (ok && go) {
         load_u(t, up);
         epilogue(t, up);
-      } else if (tid == 0) {
+      } else if (!ok) {
         atomicOr(a.flags, kErrTimeout);
       }
     }

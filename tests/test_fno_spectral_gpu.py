@@ -30,7 +30,21 @@ def rel(x, y):
 
 # (width, modes, layers, hidden, n, batch)
 SHAPES = [(32, 12, 2, 64, 64, 9), (32, 6, 2, 64, 64, 1), (64, 10, 1, 128, 64, 3), (32, 16, 1, 64, 128, 5),
-          (32, 5, 1, 64, 64, 2), (64, 24, 1, 128, 256, 1), (64, 32, 1, 128, 64, 2)]
+          (32, 5, 1, 64, 64, 2), (64, 24, 1, 128, 256, 1), (64, 32, 1, 128, 64, 2), (64, 32, 2, 128, 256, 4),
+          (32, 16, 2, 48, 128, 2)]
+
+
+def test_rows_of_several_segments():
+    """512-point rows take two segments of the transform tables, and every block
+    walks several tiles of each; inference against the oracle."""
+    W, M, n, B = 64, 32, 512, 2
+    rng = np.random.default_rng(8)
+    sh = ofno.Shapes(3, 4, W, M, 1, 128)
+    a = rng.standard_normal((B, 3, n, n)).astype(np.float32)
+    with sp.FNO(3, 4, width=W, modes=M, layers=1, hidden=128, seed=3) as f:
+        w = ofno.round_bf16(f.get_params().astype(np.float64))
+        out = f.forward(torch.from_numpy(a).cuda()).cpu().numpy()
+    assert rel(out, ofno.forward(sh, w, a.astype(np.float64))) < 2e-5
 
 
 @pytest.mark.parametrize("W,M,L,H,n,B", SHAPES)
