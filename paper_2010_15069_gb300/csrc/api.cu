@@ -560,7 +560,7 @@ cudaError_t col(spgpe_ctx *c, bool imag, const ColArgs &a) {
                                                   : launch_col_p<double>(imag, a, c->map, c->st, c->sms);
       if (e != cudaErrorNotSupported) return e;
     }
-    return c->dtype == SPGPE_C64 ? launch_col<float>(imag, a, c->st) : launch_col<double>(imag, a, c->st);
+    return c->dtype == SPGPE_C64 ? launch_col<float>(imag, a, c->st, c->sms) : launch_col<double>(imag, a, c->st, c->sms);
   });
 }
 

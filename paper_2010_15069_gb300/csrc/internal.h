@@ -148,7 +148,7 @@ template <class T, int F> cudaError_t launch_row_f(RowArgs a, cudaStream_t s);
 template <class T, int F> cudaError_t launch_row_pf(RowArgs a, cudaStream_t s, int sms);
 template <class T> LaunchShape col_shape(int nx, int ny);
 template <class T> cudaError_t launch_row(int flags, RowArgs a, cudaStream_t s);
-template <class T> cudaError_t launch_col(bool imag, ColArgs a, cudaStream_t s);
+template <class T> cudaError_t launch_col(bool imag, ColArgs a, cudaStream_t s, int sms);
 template <class T> cudaError_t launch_energy(EnergyArgs a, cudaStream_t s, int *row_blocks, int *col_blocks);
 template <class T> cudaError_t launch_norm(const void *psi, long plane, int ninst, double *partials, int blocks,
                                            cudaStream_t s);

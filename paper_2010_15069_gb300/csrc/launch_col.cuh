@@ -34,10 +34,28 @@ template <class K> cudaError_t grant_smem_c(K kern, size_t smem, int &granted) {
   return cudaSuccess;
 }
 
-template <class T, int LOGN, bool IMAG> cudaError_t col_launch_n(ColArgs a, cudaStream_t st) {
+// Columns per block of the plain column pass for a batch of ninst instances:
+// those of col_shape; in double precision, whose passes are bound by the FP64
+// units of the SMs that take part, halved (down to one 32-byte sector per row
+// and a whole warp of threads) until there is a block for every SM.  One 256^2
+// complex128 instance: 42.2 us in 64 tiles of 8 columns by TMA, 24.7 in 256 of
+// 2.  Not in single precision: 9.4 -> 10.5 us for one 256^2 instance (the
+// narrower tiles' own latency), so there the tile stays.
+template <class T> LaunchShape col_shape_spread(int nx, int ny, int ninst, int sms) {
+  LaunchShape s = col_shape<T>(nx, ny);
+  while (sizeof(T) == 8 && (long)s.blocks_x * 2 * ninst < sms && s.rows_or_cols * (int)sizeof(cx<T>) > 32 && s.threads > 32) {
+    s.rows_or_cols /= 2;
+    s.threads /= 2;
+    s.blocks_x *= 2;
+  }
+  s.smem = (size_t)col_smem_elems(ny, s.rows_or_cols, sizeof(cx<T>)) * sizeof(cx<T>);
+  return s;
+}
+
+template <class T, int LOGN, bool IMAG> cudaError_t col_launch_n(ColArgs a, cudaStream_t st, int sms) {
   constexpr int LOGE = col_loge<T>(LOGN);
   auto kern = col_pass<T, LOGN, LOGE, IMAG>;
-  const LaunchShape sh = col_shape<T>(a.nx, a.ny);
+  const LaunchShape sh = col_shape_spread<T>(a.nx, a.ny, a.ninst, sms);
   static int granted = 0;
   cudaError_t e = grant_smem_c(kern, sh.smem, granted);
   if (e != cudaSuccess) return e;
@@ -95,9 +113,9 @@ template <class T, int LOGN> cudaError_t energy_col_launch_n(EnergyArgs a, cudaS
     default: return cudaErrorInvalidValue; \
   }
 
-template <class T> cudaError_t launch_col(bool imag, ColArgs a, cudaStream_t st) {
-#define SPGPE_COL_REAL(L) col_launch_n<T, L, false>(a, st)
-#define SPGPE_COL_IMAG(L) col_launch_n<T, L, true>(a, st)
+template <class T> cudaError_t launch_col(bool imag, ColArgs a, cudaStream_t st, int sms) {
+#define SPGPE_COL_REAL(L) col_launch_n<T, L, false>(a, st, sms)
+#define SPGPE_COL_IMAG(L) col_launch_n<T, L, true>(a, st, sms)
   if (imag) {
     SPGPE_SWITCH_LOGN(a.ny, SPGPE_COL_IMAG)
   } else {
@@ -156,9 +174,12 @@ cudaError_t colp_launch_n(ColArgs a, const CUtensorMap &map, cudaStream_t st, in
   constexpr int N = 1 << LOGN, TT = N >> LOGE;
   constexpr int C = colp_cols_c<T>(LOGN, LOGE);
   if (a.nx < C) return cudaErrorNotSupported;  // narrower than one tile: the plain pass
+  const int ntiles = (a.nx / C) * 2 * a.ninst;
+  const int es = sizeof(cx<T>);
+  // double precision, tiles for part of the SMs only: the plain pass, in narrower ones (col_shape_spread)
+  if (es == 16 && ntiles < sms) return cudaErrorNotSupported;
   auto kern = col_pass_p<T, LOGN, LOGE, IMAG, C>;
   const int threads = C * TT;
-  const int es = sizeof(cx<T>);
   const size_t smem = kPipe * colp_buf_bytes(N, C, es) + (size_t)N * es +
                       colp_tw_bytes<T>(LOGN, C, Plan<LOGN, LOGE>::entries()) + kPipe * sizeof(uint64_t);
   if (smem > kMaxSmemPerBlock) return cudaErrorNotSupported;  // caller falls back to the plain pass
@@ -173,7 +194,6 @@ cudaError_t colp_launch_n(ColArgs a, const CUtensorMap &map, cudaStream_t st, in
     occ_threads = threads;
     occ_smem = smem;
   }
-  const int ntiles = (a.nx / C) * 2 * a.ninst;
   const int grid = std::max(1, std::min(ntiles, std::max(1, occ_blocks) * sms));
   a.C = C;
   kern<<<grid, threads, smem, st>>>(map, a, ntiles);
@@ -223,7 +243,7 @@ template <class T> cudaError_t launch_ref_K(const ColArgs &a, cudaStream_t st) {
 
 #define SPGPE_INSTANTIATE_COL(T)                                                              \
   template LaunchShape col_shape<T>(int, int);                                                \
-  template cudaError_t launch_col<T>(bool, ColArgs, cudaStream_t);                            \
+  template cudaError_t launch_col<T>(bool, ColArgs, cudaStream_t, int);                       \
   template cudaError_t launch_energy<T>(EnergyArgs, cudaStream_t, int *, int *);              \
   template cudaError_t launch_norm<T>(const void *, long, int, double *, int, cudaStream_t);  \
   template cudaError_t launch_residual<T>(const void *, const void *, long, int, double *, int, \

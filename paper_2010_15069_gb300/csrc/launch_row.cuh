@@ -74,19 +74,29 @@ template <class T, int LOGN, int F> cudaError_t rowp_launch_n(RowArgs a, cudaStr
   using U = RowUnit<N, E>;
   if (a.ny < U::ROWS) return cudaErrorNotSupported;  // a unit would span instances: the plain pass
   auto kern = row_pass_p<T, LOGN, LOGE, F>;
-  const int threads = rowu_block(N, E);
-  const int upb = U::WARP ? threads / 32 : 1;  // units per block
-  const size_t smem = rowu_smem(N, E, sizeof(cx<T>), Plan<LOGN, LOGE>::entries());
+  const int nunits = a.ninst * (a.ny / U::ROWS);
+  // Full blocks of warp units only once every SM gets one: a small batch is
+  // spread over the SMs instead, as few warps per block as that takes (a
+  // complex128 warp keeps its SM's FP64 unit busy by itself: one 64^2
+  // instance, 32 units, as 32 blocks of one warp instead of 4 of 8 takes 29
+  // instead of 67 us for pass A; 256^2 in complex64, 12.5 instead of 13.5 us a
+  // step).
+  const int most = rowu_block(N, E) / 32;
+  const int upb = !U::WARP ? 1 : std::max(1, std::min(most, (nunits + sms - 1) / sms));  // units per block
+  const int threads = U::WARP ? 32 * upb : rowu_block(N, E);
+  const size_t smem = U::WARP ? rowu_smem(N, E, sizeof(cx<T>), Plan<LOGN, LOGE>::entries()) -
+                                    (size_t)(most - upb) * rowu_bytes(N, U::ROWS, sizeof(cx<T>))
+                              : rowu_smem(N, E, sizeof(cx<T>), Plan<LOGN, LOGE>::entries());
   if (smem > kMaxSmemPerBlock) return cudaErrorNotSupported;
   static int granted = 0;
   cudaError_t e = grant_smem(kern, smem, granted);
   if (e != cudaSuccess) return e;
-  static int occ_blocks = -1;
+  static int occ_blocks = -1;  // of full blocks (a smaller one is not launched more than once per SM)
   if (occ_blocks < 0) {
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_blocks, kern, threads, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_blocks, kern, rowu_block(N, E),
+                                                      rowu_smem(N, E, sizeof(cx<T>), Plan<LOGN, LOGE>::entries()));
     if (e != cudaSuccess) return e;
   }
-  const int nunits = a.ninst * (a.ny / U::ROWS);
   const int grid = std::max(1, std::min((nunits + upb - 1) / upb, std::max(1, occ_blocks) * sms));
   a.rows = U::ROWS;
   kern<<<grid, threads, smem, st>>>(a, nunits);
