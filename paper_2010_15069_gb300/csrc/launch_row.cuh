@@ -84,17 +84,15 @@ template <class T, int LOGN, int F> cudaError_t rowp_launch_n(RowArgs a, cudaStr
   const int most = rowu_block(N, E) / 32;
   const int upb = !U::WARP ? 1 : std::max(1, std::min(most, (nunits + sms - 1) / sms));  // units per block
   const int threads = U::WARP ? 32 * upb : rowu_block(N, E);
-  const size_t smem = U::WARP ? rowu_smem(N, E, sizeof(cx<T>), Plan<LOGN, LOGE>::entries()) -
-                                    (size_t)(most - upb) * rowu_bytes(N, U::ROWS, sizeof(cx<T>))
-                              : rowu_smem(N, E, sizeof(cx<T>), Plan<LOGN, LOGE>::entries());
-  if (smem > kMaxSmemPerBlock) return cudaErrorNotSupported;
+  const size_t full_smem = rowu_smem(N, E, sizeof(cx<T>), Plan<LOGN, LOGE>::entries());
+  const size_t smem = U::WARP ? full_smem - (size_t)(most - upb) * rowu_bytes(N, U::ROWS, sizeof(cx<T>)) : full_smem;
+  if (full_smem > kMaxSmemPerBlock) return cudaErrorNotSupported;
   static int granted = 0;
-  cudaError_t e = grant_smem(kern, smem, granted);
+  cudaError_t e = grant_smem(kern, full_smem, granted);  // (a full block's, which the occupancy below is asked for)
   if (e != cudaSuccess) return e;
   static int occ_blocks = -1;  // of full blocks (a smaller one is not launched more than once per SM)
   if (occ_blocks < 0) {
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_blocks, kern, rowu_block(N, E),
-                                                      rowu_smem(N, E, sizeof(cx<T>), Plan<LOGN, LOGE>::entries()));
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_blocks, kern, rowu_block(N, E), full_smem);
     if (e != cudaSuccess) return e;
   }
   const int grid = std::max(1, std::min((nunits + upb - 1) / upb, std::max(1, occ_blocks) * sms));
