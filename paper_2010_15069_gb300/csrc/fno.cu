@@ -178,7 +178,9 @@ int ensure_workspace(spgpe_fno *f, int B, int n) {
   const int splits = (int)std::max<size_t>(1, P / 1024);
   size_t wmax = std::max<size_t>((size_t)f->W * f->cin, (size_t)f->W * f->W);
   wmax = std::max(wmax, std::max((size_t)f->H * f->W, (size_t)f->cout * f->H));
-  f->part_n = std::max((size_t)B * splits * wmax, (size_t)f->sms * (size_t)project_partials(f->H, f->cout));
+  // (of the general path; of the tensor-core weight gradients, a weight and a bias; of the projection)
+  f->part_n = std::max(std::max((size_t)B * splits * wmax, (size_t)2 * f->sms * (wmax + std::max(f->W, f->H))),
+                       (size_t)f->sms * (size_t)project_partials(f->H, f->cout));
   if ((r = falloc(f, &f->X1, rows * 2)) || (r = falloc(f, &f->hp, hid)) || (r = falloc(f, &f->h, hid)) ||
       (r = falloc(f, &f->dh, hid)) || (r = falloc(f, &f->dv, act)) || (r = falloc(f, &f->dv2, act)) ||
       (r = falloc(f, &f->dout, (size_t)B * f->cout * P)) || (r = falloc(f, &f->oh, spec)) ||
@@ -256,12 +258,21 @@ int read_flags(spgpe_fno *f) {
   return SPGPE_OK;
 }
 
-// grad[M][N] = sum_b sum_p A[b](m, p) Bm[b](p, n): split-K over the points,
-// partials reduced in a fixed order.
-int wgrad(spgpe_fno *f, int M, int N, long P, int B, const float *A, long sAb, const float *Bm, long sBn, long sBb,
-          float *grad) {
+// grad[M][N] = sum_b sum_p A[b](m, p) Bm[b](n, p), and (bias not null) bias[M] =
+// sum_b sum_p A[b](m, p): partial sums reduced in a fixed order.
+int wgrad(spgpe_fno *f, int M, int N, long P, int B, const float *A, long sAb, const float *Bm, long sBb, float *grad,
+          float *bias) {
+  const WeightGrad wg{M, N, B, P, A, sAb, Bm, sBb, f->part, bias != nullptr, f->d_flags};
+  if (f->tensor_cores && f->sms > 0 && weight_grad_applies(wg)) {
+    const int parts = weight_grad_parts(B, P, f->sms);
+    const long n = (long)M * N, stride = n + (bias ? M : 0);
+    FCK(f, weight_grad(wg, f->sms, f->st));
+    FCK(f, sum_parts(f->part, stride, parts, n, grad, f->st));
+    if (bias) FCK(f, sum_parts(f->part + n, stride, parts, M, bias, f->st));
+    return SPGPE_OK;
+  }
   const int splits = (int)std::max<long>(1, P / 1024);
-  GemmR g = rg(M, N, (int)P, A, false, P, 1, Bm, 1, sBn, f->part, N, 1);
+  GemmR g = rg(M, N, (int)P, A, false, P, 1, Bm, 1, P, f->part, N, 1);
   g.batch = B;
   g.sAb = sAb;
   g.sBb = sBb;
@@ -270,6 +281,7 @@ int wgrad(spgpe_fno *f, int M, int N, long P, int B, const float *A, long sAb, c
   g.sCs = (long)M * N;
   FCK(f, greal(f, g, f->st));
   FCK(f, sum_splits(f->part, (long)M * N, B * splits, grad, false, f->st));
+  if (bias) FCK(f, bias_gradient(A, B, M, P, bias, f->bscr, f->st));
   return SPGPE_OK;
 }
 
@@ -417,19 +429,17 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
     FCK(f, sum_parts(f->part, np, parts, C * H, f->g + f->oQ2, st));
     FCK(f, sum_parts(f->part + C * H, np, parts, H, f->g + f->oq1, st));
     FCK(f, sum_parts(f->part + C * H + H, np, parts, C, f->g + f->oq2, st));
-    if ((r = wgrad(f, H, W, P, B, f->dh, H * P, f->vs[f->L], P, WP, f->g + f->oQ1))) return r;
+    if ((r = wgrad(f, H, W, P, B, f->dh, H * P, f->vs[f->L], WP, f->g + f->oQ1, nullptr))) return r;
     FCK(f, project_transpose(f->dh, bfp(f, f->oQ1), f->dv, B, f->W, P, f->sms, f->d_flags, st));
   } else {
-    if ((r = wgrad(f, C, H, P, B, f->dout, C * P, f->h, P, H * P, f->g + f->oQ2))) return r;
-    FCK(f, bias_gradient(f->dout, B, C, P, f->g + f->oq2, f->bscr, st));
+    if ((r = wgrad(f, C, H, P, B, f->dout, C * P, f->h, H * P, f->g + f->oQ2, f->g + f->oq2))) return r;
     g = rg(H, P, C, bfp(f, f->oQ2), true, 1, H, f->dout, P, 1, f->dh, P, 1);
     g.batch = B;
     g.sBb = C * P;
     g.sCb = H * P;
     FCK(f, greal(f, g, st));
     FCK(f, gelu_backward(f->hp, f->dh, (long)B * H * P, st));
-    if ((r = wgrad(f, H, W, P, B, f->dh, H * P, f->vs[f->L], P, WP, f->g + f->oQ1))) return r;
-    FCK(f, bias_gradient(f->dh, B, H, P, f->g + f->oq1, f->bscr, st));
+    if ((r = wgrad(f, H, W, P, B, f->dh, H * P, f->vs[f->L], WP, f->g + f->oQ1, f->g + f->oq1))) return r;
     g = rg(W, P, H, bfp(f, f->oQ1), true, 1, W, f->dh, P, 1, f->dv, P, 1);
     g.batch = B;
     g.sBb = H * P;
@@ -440,8 +450,7 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
   for (int l = f->L - 1; l >= 0; --l) {
     // (the fused layer pass has multiplied du by the activation's derivative)
     if (l < f->L - 1 && !use_layer(f, n)) FCK(f, gelu_backward(f->us[l], du, (long)B * WP, st));
-    if ((r = wgrad(f, W, W, P, B, du, WP, f->vs[l], P, WP, f->g + f->oW[l]))) return r;
-    FCK(f, bias_gradient(du, B, W, P, f->g + f->ow[l], f->bscr, st));
+    if ((r = wgrad(f, W, W, P, B, du, WP, f->vs[l], WP, f->g + f->oW[l], f->g + f->ow[l]))) return r;
     // spectral part: doh = Ey (du Exi^T)
     float2 *doh = f->dohs[l];
     if ((r = spectrum(f, du, true, B, n, doh))) return r;
@@ -476,8 +485,7 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
     FCK(f, greal(f, g, st));
     std::swap(du, dvn);
   }
-  if ((r = wgrad(f, W, f->cin, P, B, du, WP, a, P, (long)f->cin * P, f->g + f->oP))) return r;
-  FCK(f, bias_gradient(du, B, W, P, f->g + f->op, f->bscr, st));
+  if ((r = wgrad(f, W, f->cin, P, B, du, WP, a, (long)f->cin * P, f->g + f->oP, f->g + f->op))) return r;
   if (loss) {
     std::vector<double> s((size_t)2 * B);
     FCK(f, cudaMemcpyAsync(s.data(), f->sums, s.size() * sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -55,6 +55,25 @@ cudaError_t gemm_real(const GemmR &g, cudaStream_t st);
 // for any other shape.
 bool gemm_tc_applies(const GemmR &g);
 cudaError_t gemm_real_tc(const GemmR &g, cudaStream_t st);
+// Weight and bias gradients on the tensor cores (fno_tc.cu): per CTA (of
+// weight_grad_parts), a partial dW [M][N] = sum over its points of X[b](m, p)
+// Y[b](n, p) and, with bias, db [M] = sum X[b](m, p), (M N + M) or M N floats
+// each in part, for sum_parts.  X [b][M][P], Y [b][N][P] with sample strides
+// sXb, sYb; M, N <= 128, P a multiple of 64, 16-byte aligned.
+struct WeightGrad {
+  int M, N, batch;
+  long P;
+  const float *X;
+  long sXb;
+  const float *Y;
+  long sYb;
+  float *part;
+  bool bias;
+  int *flags;
+};
+bool weight_grad_applies(const WeightGrad &g);
+int weight_grad_parts(int batch, long P, int sms);
+cudaError_t weight_grad(const WeightGrad &g, int sms, cudaStream_t st);
 cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool accumulate, cudaStream_t st);
 cudaError_t gemm_complex(const GemmC &g, cudaStream_t st);
 // Truncated Fourier transforms (fno_dft.cu) of `images` n x n fields with the

@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(32 * kGradModes) mix_grad(const float2 *__rest
   __syncthreads();
   load(d);
   __syncthreads();
-#pragma unroll 2
+#pragma unroll 4
   for (int o = 0; o < W; ++o) {
     const long p = (m * W + o) * W + NC * lane;
     using V = Cols<NC>;

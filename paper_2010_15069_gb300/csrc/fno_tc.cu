@@ -215,145 +215,168 @@ cudaError_t launch_tc(const GemmR &g, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Weight gradients on the tensor cores: part[b splits + s](m, n) =
-// sum over points p of split s of X[b](m, p) Y[b](n, p), m < M, n < N, both
-// operands float32 with unit stride along p (the K dimension of the MMA).  Each
-// operand is split into two bfloat16 terms (x = h + l, 16 significant bits),
-// and the three products h h', h l', l h' are accumulated (the dropped l l' is
-// below 2^-16 of the result).  The MMA tile is 128 rows of X (M <= MR = 64 or
-// 128; the rows from M on stay zero) by NC = 16, 64 or 128 rows of Y (N <= NC,
-// likewise).  One CTA per (sample, split), its 64-point blocks streamed
-// through registers one block ahead of the MMAs.
+// Weight gradients on the tensor cores: dW[m][n] = sum over samples and points
+// of X[b](m, p) Y[b](n, p), m < M, n < N, both operands float32 with unit
+// stride along p (the K dimension of the MMA), and the bias gradient db[m] =
+// sum X[b](m, p) beside it (X is on its way through the registers anyway).
+// Each operand is split into two bfloat16 terms (x = h + l, 16 significant
+// bits), and the three products h h', h l', l h' are accumulated (the dropped
+// l l' is below 2^-16 of the result).  The MMA tile is 128 rows of X (M <= MR =
+// 64 or 128; the rows from M on stay zero) by NC = 16, 64 or 128 rows of Y (N <=
+// NC, likewise); the terms of Y lie side by side, so that X's h term meets both
+// in one MMA of 2 NC columns.  Persistent CTAs each take a run of 64-point
+// blocks and leave one partial sum; two operand buffers, the next block's
+// values in registers while the tensor cores work.  Bound by the one read of
+// both operands.
 template <int MR, int NC> struct WgSmem {
   static constexpr size_t kA = (size_t)kTcRows * kRowBytes;  // one term of X
   static constexpr size_t kB = (size_t)NC * kRowBytes;       // one term of Y
-  static constexpr size_t kBytes = 1024 + 2 * kA + 2 * kB + 16;
+  static constexpr size_t kStage = 2 * kA + 2 * kB;
+  static constexpr size_t kBytes = 1024 + 2 * kStage + 64;
 };
 
+constexpr int kWgThreads = 256;
+
 template <int MR, int NC>
-__global__ void __launch_bounds__(128) gemm_tc_wgrad(int M, int N, int splits, int ks, const float *__restrict__ X,
-                                                     long sXm, long sXb, const float *__restrict__ Y, long sYn,
-                                                     long sYb, float *part, long sPs, int *flags) {
+__global__ void __launch_bounds__(kWgThreads, 2) gemm_tc_wgrad(int M, int N, int nblk, int blocks_per_sample,
+                                                            const float *__restrict__ X, long sXm, long sXb,
+                                                            const float *__restrict__ Y, long sYn, long sYb, float *part,
+                                                            long sPs, int with_bias, int *flags) {
   using S = WgSmem<MR, NC>;
-  constexpr uint32_t kCols = NC < 32 ? 32 : NC;  // TMEM allocations are powers of two from 32 columns
-  constexpr int CH = (MR + NC) * 8 / 128;  // 16-byte chunks of one 64-point block per thread
+  constexpr uint32_t kCols = 2 * NC < 32 ? 32 : 2 * NC;
+  constexpr int CH = (MR + NC) * 8 / kWgThreads;  // 16-byte runs of one 64-point block per thread
+  constexpr int CHX = MR * 8 / kWgThreads;        // those of X
+  static_assert((MR + NC) * 8 % kWgThreads == 0 || NC == 16, "whole runs per thread");
+  constexpr int CHT = ((MR + NC) * 8 + kWgThreads - 1) / kWgThreads;
   extern __shared__ unsigned char smem_raw[];
   unsigned char *sm =
       reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  unsigned char *sA = sm, *sB = sm + 2 * S::kA;
-  uint64_t *bar = reinterpret_cast<uint64_t *>(sB + 2 * S::kB);
-  uint32_t *slot = reinterpret_cast<uint32_t *>(bar + 1);
+  uint64_t *mma = reinterpret_cast<uint64_t *>(sm + 2 * S::kStage);
+  uint32_t *slot = reinterpret_cast<uint32_t *>(mma + 2);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int b = blockIdx.x / splits, sp = blockIdx.x - b * splits;
-  const long k0 = (long)sp * ks;
-  const float *xb = X + b * sXb + k0, *yb = Y + b * sYb + k0;
+  (void)CH;
+  const int b0 = (int)((long)blockIdx.x * nblk / gridDim.x), b1 = (int)((long)(blockIdx.x + 1) * nblk / gridDim.x);
 
   if (warp == 0) {
     tmem_alloc(slot, kCols);
     tmem_relinquish();
   }
   if (tid == 0) {
-    mbar_init(bar, 1);
+    mbar_init(&mma[0], 1);
+    mbar_init(&mma[1], 1);
     mbar_fence_init();
   }
   // rows M..127 of both X terms and N..NC-1 of both Y terms stay zero
-  for (int e = tid; e < (kTcRows - M) * 8; e += blockDim.x) {
-    const int r = M + e / 8, c = e % 8;
-    *reinterpret_cast<uint4 *>(sA + sw128(r, c)) = make_uint4(0, 0, 0, 0);
-    *reinterpret_cast<uint4 *>(sA + S::kA + sw128(r, c)) = make_uint4(0, 0, 0, 0);
-  }
-  for (int e = tid; e < (NC - N) * 8; e += blockDim.x) {
-    const int r = N + e / 8, c = e % 8;
-    *reinterpret_cast<uint4 *>(sB + sw128(r, c)) = make_uint4(0, 0, 0, 0);
-    *reinterpret_cast<uint4 *>(sB + S::kB + sw128(r, c)) = make_uint4(0, 0, 0, 0);
+  for (int s = 0; s < 2; ++s) {
+    unsigned char *sA = sm + s * S::kStage, *sB = sA + 2 * S::kA;
+    for (int e = tid; e < (kTcRows - M) * 8; e += kWgThreads) {
+      const int r = M + e / 8, c = e % 8;
+      *reinterpret_cast<uint4 *>(sA + sw128(r, c)) = make_uint4(0, 0, 0, 0);
+      *reinterpret_cast<uint4 *>(sA + S::kA + sw128(r, c)) = make_uint4(0, 0, 0, 0);
+    }
+    for (int e = tid; e < (NC - N) * 8; e += kWgThreads) {
+      const int r = N + e / 8, c = e % 8;
+      *reinterpret_cast<uint4 *>(sB + sw128(r, c)) = make_uint4(0, 0, 0, 0);
+      *reinterpret_cast<uint4 *>(sB + S::kB + sw128(r, c)) = make_uint4(0, 0, 0, 0);
+    }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *slot;
-  constexpr uint32_t idesc = idesc_bf16(kTcRows, NC);
-  // chunk q of a block: rows 0..MR-1 of X then rows of Y, 8 chunks (64 points) per row
-  float4 xr[CH][2];
+  // run q of a block: rows 0..MR-1 of X then rows of Y, 8 runs (64 points) per row
+  float4 xr[CHT][2];
+  float bsum[CHX];
+#pragma unroll
+  for (int q = 0; q < CHX; ++q) bsum[q] = 0.f;
   // valid rows only (the others keep their zeros)
   auto valid = [&](int r) { return r < MR ? r < M : r - MR < N; };
-  auto load = [&](long kk) {
+  auto load = [&](int blk) {
+    const int b = blk / blocks_per_sample;
+    const long k0 = (long)(blk - b * blocks_per_sample) * kKBlock;
+    const float *xb = X + b * sXb + k0, *yb = Y + b * sYb + k0;
 #pragma unroll
-    for (int q = 0; q < CH; ++q) {
-      const int e = tid + q * 128, r = e / 8, c = e % 8;
+    for (int q = 0; q < CHT; ++q) {
+      const int e = tid + q * kWgThreads, r = e / 8, c = e % 8;
       if (valid(r)) {
-        const float *src = r < MR ? xb + r * sXm + kk + 8 * c : yb + (r - MR) * sYn + kk + 8 * c;
+        const float *src = r < MR ? xb + r * sXm + 8 * c : yb + (r - MR) * sYn + 8 * c;
         xr[q][0] = *reinterpret_cast<const float4 *>(src);
         xr[q][1] = *reinterpret_cast<const float4 *>(src + 4);
       }
     }
   };
-  auto split2 = [&](float v, __nv_bfloat16 &h, __nv_bfloat16 &l) {
-    h = __float2bfloat16_rn(v);
-    l = __float2bfloat16_rn(v - __bfloat162float(h));
-  };
   bool ok = true;
-  const int nblk = ks / kKBlock;
-  load(0);
-  for (int blk = 0; blk < nblk && ok; ++blk) {
+  if (b0 < b1) load(b0);
+  int i = 0;
+  for (int blk = b0; blk < b1 && ok; ++blk, ++i) {
+    const int s = i & 1;
+    unsigned char *sA = sm + s * S::kStage, *sB = sA + 2 * S::kA;
+    if (i >= 2) ok = mbar_wait_bounded(&mma[s], (uint32_t)(((i >> 1) - 1) & 1));
 #pragma unroll
-    for (int q = 0; q < CH; ++q) {
-      const int e = tid + q * 128, r = e / 8, c = e % 8;
+    for (int q = 0; q < CHT; ++q) {
+      const int e = tid + q * kWgThreads, r = e / 8, c = e % 8;
       if (!valid(r)) continue;
       const float v[8] = {xr[q][0].x, xr[q][0].y, xr[q][0].z, xr[q][0].w,
                           xr[q][1].x, xr[q][1].y, xr[q][1].z, xr[q][1].w};
+      if (q < CHX) bsum[q < CHX ? q : 0] += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
       uint32_t hw[4], lw[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        __nv_bfloat16 h0, l0, h1, l1;
-        split2(v[2 * i], h0, l0);
-        split2(v[2 * i + 1], h1, l1);
-        hw[i] = pack_bf16(h0, h1);
-        lw[i] = pack_bf16(l0, l1);
+      for (int j = 0; j < 4; ++j) {
+        hw[j] = cvt_bf16x2(v[2 * j], v[2 * j + 1]);
+        lw[j] = cvt_bf16x2(v[2 * j] - __uint_as_float(hw[j] << 16), v[2 * j + 1] - __uint_as_float(hw[j] & 0xffff0000u));
       }
       unsigned char *dst = r < MR ? sA + sw128(r, c) : sB + sw128(r - MR, c);
       const size_t term = r < MR ? S::kA : S::kB;
       *reinterpret_cast<uint4 *>(dst) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
       *reinterpret_cast<uint4 *>(dst + term) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
     }
+    if (blk + 1 < b1) load(blk + 1);
     fence_proxy_async();
-    __syncthreads();
+    ok = __syncthreads_and(ok);
     if (tid == 0) {
+      // (the commit follows in any case, so that every wait ends)
       tc_fence_after();
-      const uint64_t ah = sw128_desc(sA), al = sw128_desc(sA + S::kA);
-      const uint64_t bh = sw128_desc(sB), bl = sw128_desc(sB + S::kB);
+      const uint64_t ah = sw128_desc(sA), al = sw128_desc(sA + S::kA), bd = sw128_desc(sB);
+      if (ok)
 #pragma unroll
-      for (int kk = 0; kk < kKBlock / 16; ++kk) {
-        umma_bf16(tmem, ah + 2 * kk, bh + 2 * kk, idesc, (blk | kk) != 0);
-        umma_bf16(tmem, ah + 2 * kk, bl + 2 * kk, idesc, 1);
-        umma_bf16(tmem, al + 2 * kk, bh + 2 * kk, idesc, 1);
-      }
-      umma_commit(bar);
-    }
-    if (blk + 1 < nblk) load((long)(blk + 1) * kKBlock);
-    // the next block's operands go into the same buffers: wait for these MMAs
-    ok = mbar_wait_bounded(bar, (uint32_t)(blk & 1));
-    if (!__syncthreads_and(ok)) {
-      if (tid == 0) atomicOr(flags, kErrTimeout);
-      mbar_wait_bounded(bar, (uint32_t)(blk & 1));
-      ok = false;
+        for (int kk = 0; kk < kKBlock / 16; ++kk) {
+          umma_bf16(tmem, ah + 2 * kk, bd + 2 * kk, idesc_bf16(kTcRows, 2 * NC), (i | kk) != 0);
+          umma_bf16(tmem, al + 2 * kk, bd + 2 * kk, idesc_bf16(kTcRows, NC), 1);
+        }
+      umma_commit(&mma[s]);
     }
   }
-  if (ok) {
-    tc_fence_after();
-    // rows 0..M-1 of the accumulator, columns 0..N-1: lanes of the first warps
-    if (32 * warp < M) {
-      const int m = 32 * warp + lane;
-      float *out = part + (long)blockIdx.x * sPs + (long)m * N;
+  // every MMA issued is complete before the buffers go (and the barrier brings
+  // the lanes together for the tensor-memory loads)
+  if (i > 0) ok = mbar_wait_bounded(&mma[(i - 1) & 1], (uint32_t)(((i - 1) >> 1) & 1)) && ok;
+  ok = __syncthreads_and(ok);
+  if (!ok && tid == 0) atomicOr(flags, kErrTimeout);
+  tc_fence_after();
+  // rows 0..M-1 of the accumulator, columns n and NC + n: warps 0-3 and 4-7
+  // hold the same lanes and take alternate groups of columns
+  float *out = part + (long)blockIdx.x * sPs;
+  if (ok && 32 * (warp & 3) < M) {
+    const int m = 32 * (warp & 3) + lane;
 #pragma unroll
-      for (int c0 = 0; c0 < NC; c0 += 16) {
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0, v);
-        tmem_ld_wait();
-        if (m < M)
+    for (int c0 = 8 * (warp >> 2); c0 < NC; c0 += 16) {
+      float v[8], u[8];
+      tmem_ld8(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, v);
+      tmem_ld8(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(NC + c0), u);
+      tmem_ld_wait();
+      if (m < M)
 #pragma unroll
-          for (int i = 0; i < 16; ++i)
-            if (c0 + i < N) out[c0 + i] = v[i];
-      }
+        for (int j = 0; j < 8; ++j)
+          if (c0 + j < N) out[(long)m * N + c0 + j] = i > 0 ? v[j] + u[j] : 0.f;
+    }
+  }
+  if (with_bias) {  // 8 lanes hold a row
+#pragma unroll
+    for (int q = 0; q < CHX; ++q) {
+      float v = bsum[q];
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      const int r = (tid + q * kWgThreads) / 8;
+      if ((tid & 7) == 0 && r < M) out[(long)M * N + r] = v;
     }
   }
   tc_fence_before();
@@ -365,35 +388,44 @@ __global__ void __launch_bounds__(128) gemm_tc_wgrad(int M, int N, int splits, i
 }
 
 template <int MR, int NC>
-cudaError_t launch_wgrad(const GemmR &g, cudaStream_t st) {
+cudaError_t launch_wgrad(const WeightGrad &g, int grid, cudaStream_t st) {
   auto kern = gemm_tc_wgrad<MR, NC>;
-  const size_t smem = WgSmem<MR, NC>::kBytes;
-  static int granted = 0;
+  constexpr size_t smem = WgSmem<MR, NC>::kBytes;
+  static bool granted = false;
   if (!granted) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    granted = 1;
+    granted = true;
   }
-  kern<<<g.batch * g.splits, 128, smem, st>>>(g.M, g.N, g.splits, g.K / g.splits, static_cast<const float *>(g.A),
-                                              g.sAm, g.sAb, g.B, g.sBn, g.sBb, g.C, g.sCs, g.flags);
+  const int bps = (int)(g.P / kKBlock);
+  kern<<<grid, kWgThreads, smem, st>>>(g.M, g.N, g.batch * bps, bps, g.X, g.P, g.sXb, g.Y, g.P, g.sYb, g.part,
+                                       (long)g.M * g.N + (g.bias ? g.M : 0), g.bias ? 1 : 0, g.flags);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-namespace {
-// split-K weight gradients of two float32 operands with unit stride along K
-bool wgrad_applies(const GemmR &g) {
-  return !g.a_bf16 && g.flags && g.partial && g.sAk == 1 && g.sBk == 1 && g.sCm == g.N && g.sCn == 1 &&
-         g.sCs == (long)g.M * g.N && g.M >= 1 && g.M <= 128 && g.N >= 1 && g.N <= 128 && g.splits >= 1 &&
-         g.K % g.splits == 0 && (g.K / g.splits) % kKBlock == 0 && g.sAm % 4 == 0 && g.sBn % 4 == 0 &&
-         g.sAb % 4 == 0 && g.sBb % 4 == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0 &&
-         (reinterpret_cast<uintptr_t>(g.B) & 15) == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
+bool weight_grad_applies(const WeightGrad &g) {
+  return g.M >= 1 && g.M <= 128 && g.N >= 1 && g.N <= 128 && g.P % kKBlock == 0 && g.sXb % 4 == 0 && g.sYb % 4 == 0 &&
+         (reinterpret_cast<uintptr_t>(g.X) & 15) == 0 && (reinterpret_cast<uintptr_t>(g.Y) & 15) == 0;
 }
-}  // namespace
+
+int weight_grad_parts(int batch, long P, int sms) { return (int)std::max<long>(1, std::min<long>(2L * sms, batch * (P / kKBlock))); }
+
+cudaError_t weight_grad(const WeightGrad &g, int sms, cudaStream_t st) {
+  const int grid = weight_grad_parts(g.batch, g.P, sms);
+  cudaError_t e;
+  if (g.M <= 64) {
+    if (g.N <= 16) e = launch_wgrad<64, 16>(g, grid, st);
+    else e = g.N <= 64 ? launch_wgrad<64, 64>(g, grid, st) : launch_wgrad<64, 128>(g, grid, st);
+  } else {
+    if (g.N <= 16) e = launch_wgrad<128, 16>(g, grid, st);
+    else e = g.N <= 64 ? launch_wgrad<128, 64>(g, grid, st) : launch_wgrad<128, 128>(g, grid, st);
+  }
+  return e;
+}
 
 bool gemm_tc_applies(const GemmR &g) {
-  if (wgrad_applies(g)) return true;
   return g.a_bf16 && g.flags && !g.partial && g.splits == 1 && g.alpha == 1.f && g.sAb == 0 && g.sBn == 1 &&
          g.sCn == 1 && (g.M == 64 || g.M == 128) && (g.K == 64 || g.K == 128) && g.N % kTcRows == 0 &&
          g.N >= kTcRows;
@@ -401,14 +433,6 @@ bool gemm_tc_applies(const GemmR &g) {
 
 cudaError_t gemm_real_tc(const GemmR &g, cudaStream_t st) {
   if (!gemm_tc_applies(g)) return cudaErrorNotSupported;
-  if (wgrad_applies(g)) {
-    if (g.M <= 64) {
-      if (g.N <= 16) return launch_wgrad<64, 16>(g, st);
-      return g.N <= 64 ? launch_wgrad<64, 64>(g, st) : launch_wgrad<64, 128>(g, st);
-    }
-    if (g.N <= 16) return launch_wgrad<128, 16>(g, st);
-    return g.N <= 64 ? launch_wgrad<128, 64>(g, st) : launch_wgrad<128, 128>(g, st);
-  }
   if (g.M == 64) return g.K == 64 ? launch_tc<64, 1>(g, st) : launch_tc<64, 2>(g, st);
   return g.K == 64 ? launch_tc<128, 1>(g, st) : launch_tc<128, 2>(g, st);
 }
