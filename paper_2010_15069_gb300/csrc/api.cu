@@ -92,6 +92,7 @@ struct spgpe_ctx {
   bool persistent_row = true;
   bool persistent_col = true;
   bool warp_col = true;  // the warp-local column pass where it applies (ny = 256, complex64)
+  bool overlap = true;   // passes may start before the one before them ends (launch_pdl); not in a size class
   int host_chunks = 8;   // chunks of instances a host batch goes through (copies overlap steps)
   const void *map_psi = nullptr, *map_sw_psi = nullptr;
   int map_ninst = 0, map_sw_ninst = 0;
@@ -389,6 +390,7 @@ RowArgs row_args(spgpe_ctx *c, void *psi, double dt) {
   a.nx = c->nx;
   a.ny = c->ny;
   a.ninst = c->ninst;
+  a.overlap = c->overlap ? 1 : 0;
   return a;
 }
 
@@ -441,6 +443,7 @@ ColArgs col_args(spgpe_ctx *c, void *psi) {
   a.nx = c->nx;
   a.ny = c->ny;
   a.ninst = c->ninst;
+  a.overlap = c->overlap ? 1 : 0;
   return a;
 }
 
@@ -1075,6 +1078,7 @@ int spgpe_init_multi(spgpe_ctx **out, int nclass, const int *nx, const int *ny, 
       return bail(r, g_init_error);
     }
     kc->own_stream = true;
+    kc->overlap = false;
     c->cls.push_back(kc);
     if (cudaEventCreateWithFlags(&kc->join_ev, cudaEventDisableTiming) != cudaSuccess)
       return bail(SPGPE_ECUDA, "cudaEventCreate failed");
@@ -1510,6 +1514,7 @@ int ensure_twin(spgpe_ctx *c) {
     t->persistent_row = c->persistent_row;
     t->persistent_col = c->persistent_col;
     t->warp_col = c->warp_col;
+    t->overlap = c->overlap;
     c->twin = t;
   }
   spgpe_ctx *t = c->twin;

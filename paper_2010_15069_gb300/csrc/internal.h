@@ -67,6 +67,8 @@ struct RowArgs {
   const int *active;      // [ninst] nonzero: step this instance (null: all); frozen instances are skipped
   int *flags;             // bit 0: non-finite or zero norm met
   int nx, ny, ninst, rows;
+  int overlap;            // the pass may start before the one before it ends
+  int pdl_early;          // the next kernel may start at once (set by the launcher)
 };
 
 // Arguments of the fused column pass (y direction, one component per block).
@@ -84,6 +86,7 @@ struct ColArgs {
   // predicted one, written by the row pass before); null: no such factor.
   const void *cfac;
   int nx, ny, ninst, C;
+  int overlap, pdl_early; // as in RowArgs
 };
 
 // Energy passes.

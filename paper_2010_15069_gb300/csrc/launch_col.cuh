@@ -60,8 +60,8 @@ template <class T, int LOGN, bool IMAG> cudaError_t col_launch_n(ColArgs a, cuda
   cudaError_t e = grant_smem_c(kern, sh.smem, granted);
   if (e != cudaSuccess) return e;
   a.C = sh.rows_or_cols;
-  kern<<<dim3(sh.blocks_x, 2, a.ninst), sh.threads, sh.smem, st>>>(a);
-  return cudaGetLastError();
+  a.pdl_early = a.overlap && sizeof(T) == 4 && (long)sh.blocks_x * 2 * a.ninst <= sms;
+  return launch_pdl(a.overlap, kern, dim3(sh.blocks_x, 2, a.ninst), sh.threads, sh.smem, st, a);
 }
 
 template <class T, int LOGN> cudaError_t energy_launch_n(EnergyArgs a, cudaStream_t st, int *rb, int *cb) {
@@ -196,8 +196,8 @@ cudaError_t colp_launch_n(ColArgs a, const CUtensorMap &map, cudaStream_t st, in
   }
   const int grid = std::max(1, std::min(ntiles, std::max(1, occ_blocks) * sms));
   a.C = C;
-  kern<<<grid, threads, smem, st>>>(map, a, ntiles);
-  return cudaGetLastError();
+  a.pdl_early = a.overlap && sizeof(T) == 4 && grid <= sms;
+  return launch_pdl(a.overlap, kern, dim3(grid), threads, smem, st, map, a, ntiles);
 }
 
 template <class T> cudaError_t launch_col_p(bool imag, ColArgs a, const CUtensorMap &map, cudaStream_t st,
@@ -226,8 +226,8 @@ template <bool IMAG> cudaError_t colw_launch(ColArgs a, const CUtensorMap &map, 
   const int ntiles = (a.nx / kColW_C) * 2 * a.ninst;
   const int grid = std::max(1, std::min(ntiles, std::max(1, occ) * sms));
   a.C = kColW_C;
-  kern<<<grid, 256, smem, st>>>(map, a, ntiles);
-  return cudaGetLastError();
+  a.pdl_early = a.overlap && grid <= sms;
+  return launch_pdl(a.overlap, kern, dim3(grid), 256, smem, st, map, a, ntiles);
 }
 
 template <class T> cudaError_t launch_col_w(bool imag, ColArgs a, const CUtensorMap &map, cudaStream_t st, int sms) {

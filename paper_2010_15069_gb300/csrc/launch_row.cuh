@@ -44,8 +44,7 @@ template <class T, int LOGN, int F> cudaError_t row_launch_n(RowArgs a, cudaStre
     attr_set = (int)sh.smem;
   }
   a.rows = sh.rows_or_cols;
-  kern<<<dim3(sh.blocks_x, a.ninst), sh.threads, sh.smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(a.overlap, kern, dim3(sh.blocks_x, a.ninst), sh.threads, sh.smem, st, a);
 }
 
 // One flag combination, every row length (instantiated per flag group in
@@ -97,8 +96,8 @@ template <class T, int LOGN, int F> cudaError_t rowp_launch_n(RowArgs a, cudaStr
   }
   const int grid = std::max(1, std::min((nunits + upb - 1) / upb, std::max(1, occ_blocks) * sms));
   a.rows = U::ROWS;
-  kern<<<grid, threads, smem, st>>>(a, nunits);
-  return cudaGetLastError();
+  a.pdl_early = a.overlap && sizeof(T) == 4 && grid <= sms;
+  return launch_pdl(a.overlap, kern, dim3(grid), threads, smem, st, a, nunits);
 }
 
 template <class T, int F> cudaError_t launch_row_pf(RowArgs a, cudaStream_t st, int sms) {
