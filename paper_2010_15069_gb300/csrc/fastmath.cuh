@@ -146,6 +146,16 @@ __device__ __forceinline__ void shear_consts_2h_small(float h, float &t, float &
                     -1.3333333333f), 2.0f);
 }
 
+// The magnitude of a double as a float, rounded toward zero by at most 2^-20
+// relative (below 2^-126: zero; not finite: infinity), with integer
+// instructions: an FP64 conversion runs at the FP64 rate.
+__device__ __forceinline__ float magnitude_f(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  const int e = hi - ((1023 - 127) << 20);                    // exponent rebiased
+  if (hi >= ((1023 + 128) << 20)) return __int_as_float(0x7f800000);
+  return e < (1 << 20) ? 0.f : __int_as_float(e << 3);
+}
+
 // Double precision: the CUDA math library.
 __device__ __forceinline__ void shear_consts_2h(double h, double &t, double &s, bool &neg) {
   double sh, ch;
@@ -166,9 +176,29 @@ __device__ __forceinline__ void shear_consts_2h(double h, double &t, double &s, 
     neg = (((long long)n) & 1) != 0;
   }
 }
-__device__ __forceinline__ void shear_consts_2h_small(double h, double &t, double &s) {
-  bool neg;
-  shear_consts_2h(h, t, s, neg);
+// Series in double precision for callers that know the bound for a whole warp,
+// as the single-precision ones (the library's sincos and a division cost
+// several times as many FP64 instructions, and these passes are bound by
+// them): the first omitted terms are below 1e-17 relative.
+__device__ __forceinline__ void shear_consts_2h_tiny(double h, double &t, double &s) {  // |h| < 1/64
+  const double h2 = h * h;
+  t = h * fma(h2, fma(h2, fma(h2, fma(h2, 62.0 / 2835, 17.0 / 315), 2.0 / 15), 1.0 / 3), 1.0);
+  s = h * fma(h2, fma(h2, fma(h2, -8.0 / 315, 4.0 / 15), -4.0 / 3), 2.0);
+}
+__device__ __forceinline__ void shear_consts_2h_small(double h, double &t, double &s) {  // |h| < 1/8
+  const double h2 = h * h;
+  double p = fma(h2, 929569.0 / 638512875, 21844.0 / 6081075);
+  p = fma(h2, p, 1382.0 / 155925);
+  p = fma(h2, p, 62.0 / 2835);
+  p = fma(h2, p, 17.0 / 315);
+  p = fma(h2, p, 2.0 / 15);
+  p = fma(h2, p, 1.0 / 3);
+  t = h * fma(h2, p, 1.0);
+  double q = fma(h2, -8.0 / 155925, 4.0 / 2835);
+  q = fma(h2, q, -8.0 / 315);
+  q = fma(h2, q, 4.0 / 15);
+  q = fma(h2, q, -4.0 / 3);
+  s = h * fma(h2, q, 2.0);
 }
 
 // ln 2 = A + B, A with 12 significant bits (k * A exact for |k| < 2^12).
@@ -234,9 +264,33 @@ __device__ __forceinline__ float expm1_quarter(float x) {
   return fmaf(x * x, p, x);
 }
 
-// Double precision: the CUDA math library.
-__device__ __forceinline__ double expm1_small(double x) { return expm1(x); }
-__device__ __forceinline__ double expm1_quarter(double x) { return expm1(x); }
+// Double precision, for callers that know the bound for a whole warp: Taylor
+// series to x^13/13! for |x| < 1/4 and to x^9/9! for |x| < 1/32 (first omitted
+// term below 1e-17 relative); beyond, the CUDA math library.
+__device__ __forceinline__ double expm1_small(double x) {  // |x| < 1/4
+  double p = fma(x, 1.0 / 6227020800.0, 1.0 / 479001600.0);
+  p = fma(x, p, 1.0 / 39916800.0);
+  p = fma(x, p, 1.0 / 3628800.0);
+  p = fma(x, p, 1.0 / 362880.0);
+  p = fma(x, p, 1.0 / 40320.0);
+  p = fma(x, p, 1.0 / 5040.0);
+  p = fma(x, p, 1.0 / 720.0);
+  p = fma(x, p, 1.0 / 120.0);
+  p = fma(x, p, 1.0 / 24.0);
+  p = fma(x, p, 1.0 / 6.0);
+  p = fma(x, p, 0.5);
+  return fma(x * x, p, x);
+}
+__device__ __forceinline__ double expm1_quarter(double x) {  // |x| < 1/32 (the first tier in double precision)
+  double p = fma(x, 1.0 / 362880.0, 1.0 / 40320.0);
+  p = fma(x, p, 1.0 / 5040.0);
+  p = fma(x, p, 1.0 / 720.0);
+  p = fma(x, p, 1.0 / 120.0);
+  p = fma(x, p, 1.0 / 24.0);
+  p = fma(x, p, 1.0 / 6.0);
+  p = fma(x, p, 0.5);
+  return fma(x * x, p, x);
+}
 __device__ __forceinline__ void expi2_m1(double h, double &wre, double &wim) {
   double s, c;
   sincos(h, &s, &c);

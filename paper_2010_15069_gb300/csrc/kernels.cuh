@@ -109,19 +109,18 @@ __device__ __forceinline__ double expm1_general(double x) { return expm1(x); }
 // exp(-tau V) (1 + expm1(-tau g rho)).
 // TIER (the caller has checked it for every point of the warp): real time
 // 0: |h| < 1/64, 1: |h| < 1/8; imaginary time (h the interaction exponent)
-// 0: |h| < 1/4, 1: |h| < 1/2; so the series need no range reduction; 2: any
-// phase.  FP64 always takes the library functions.
+// 0: |h| < 1/4, 1: |h| < 1/2 (double precision: 1/32 and 1/4); so the series
+// need no range reduction; 2: any phase.
 template <bool IMAG, int TIER = 2, class T>
 __device__ __forceinline__ void opD(cx<T> &u, cx<T> &d, T vu, T vd, T gh11, T gh22, T gh12) {
-  constexpr bool F32 = sizeof(T) == 4;
   const T ru = d_fma(u.re, u.re, u.im * u.im), rd = d_fma(d.re, d.re, d.im * d.im);
   if constexpr (IMAG) {
     const T hu = d_fma(gh12, rd, gh11 * ru), hd = d_fma(gh12, ru, gh22 * rd);
     T fu, fd;
-    if constexpr (F32 && TIER == 0) {
+    if constexpr (TIER == 0) {
       fu = expm1_quarter(hu);
       fd = expm1_quarter(hd);
-    } else if constexpr (F32 && TIER == 1) {
+    } else if constexpr (TIER == 1) {
       fu = expm1_small(hu);
       fd = expm1_small(hd);
     } else {
@@ -137,10 +136,10 @@ __device__ __forceinline__ void opD(cx<T> &u, cx<T> &d, T vu, T vd, T gh11, T gh
     // the phases exp(-i tau e) as three-shear rotations by 2 h
     // (determinant one: no systematic change of |psi| from rounded constants)
     T tu, su, td, sd;
-    if constexpr (F32 && TIER == 0) {
+    if constexpr (TIER == 0) {
       shear_consts_2h_tiny(hu, tu, su);
       shear_consts_2h_tiny(hd, td, sd);
-    } else if constexpr (F32 && TIER == 1) {
+    } else if constexpr (TIER == 1) {
       shear_consts_2h_small(hu, tu, su);
       shear_consts_2h_small(hd, td, sd);
     } else {
@@ -444,30 +443,44 @@ __device__ __forceinline__ void r_apply(cx<T> (&pu)[K], cx<T> (&pd)[K], int t, i
   // |V +- delta/2| of the instance and G = max(|g11|, |g22|) + |g12|;
   // rho_tot = |u|^2 + |d|^2 at a point is left unchanged by real-time R (5 %
   // margin for the imaginary-time X).
-  T rmax = T(0);
-#pragma unroll
-  for (int j = 0; j < K; ++j) rmax = fmax(rmax, d_fma(pu[j].re, pu[j].re, pu[j].im * pu[j].im) +
-                                                    d_fma(pd[j].re, pd[j].re, pd[j].im * pd[j].im));
-  // (the lagged pass scales the densities between R_end and R_start by the
-  // squared predicted scale)
-  if constexpr ((F & F_LAG) != 0) rmax *= fmax(T(1), fmax(su * su, sd * sd));
   // (imaginary time: the potential factors come from tables, so only the
-  // interaction exponent is bounded; real time: the whole phase)
-  const T hb = fabs(htau) * ((IMAG ? T(0) : gp[3]) + gmax * T(1.05) * rmax);
-  const bool small = __all_sync(mask, hb < (IMAG ? T(0.5) : T(0.125)));
-  const bool tiny = __all_sync(mask, hb < (IMAG ? T(0.25) : T(0.015625)));
+  // interaction exponent is bounded; real time: the whole phase.  The lagged
+  // pass scales the densities between R_end and R_start by the squared
+  // predicted scale.)  Double precision bounds it in single precision, with
+  // the magnitudes from integer instructions: the 5 % cover the rounding.
+  float hb;
+  if constexpr (sizeof(T) == 4) {
+    T rmax = T(0);
+#pragma unroll
+    for (int j = 0; j < K; ++j) rmax = fmax(rmax, d_fma(pu[j].re, pu[j].re, pu[j].im * pu[j].im) +
+                                                      d_fma(pd[j].re, pd[j].re, pd[j].im * pd[j].im));
+    if constexpr ((F & F_LAG) != 0) rmax *= fmax(T(1), fmax(su * su, sd * sd));
+    hb = fabs(htau) * ((IMAG ? T(0) : gp[3]) + gmax * T(1.05) * rmax);
+  } else {
+    float rmax = 0.f;
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      const float a0 = magnitude_f(pu[j].re), a1 = magnitude_f(pu[j].im), b0 = magnitude_f(pd[j].re), b1 = magnitude_f(pd[j].im);
+      rmax = fmaxf(rmax, fmaf(a0, a0, a1 * a1) + fmaf(b0, b0, b1 * b1));
+    }
+    if constexpr ((F & F_LAG) != 0) {
+      const float fu = magnitude_f(su), fd = magnitude_f(sd);
+      rmax *= fmaxf(1.f, fmaxf(fu * fu, fd * fd) * 1.00001f);
+    }
+    hb = magnitude_f(htau) * 1.00001f * ((IMAG ? 0.f : magnitude_f(gp[3]) * 1.00001f) + magnitude_f(gmax) * 1.05f * rmax);
+    if (!(rmax < 1e30f)) hb = 1e30f;  // not finite: fmaxf drops a NaN, the library functions pass it on
+  }
+  constexpr float kSmall = IMAG ? (sizeof(T) == 4 ? 0.5f : 0.25f) : 0.125f;
+  constexpr float kTiny = IMAG ? (sizeof(T) == 4 ? 0.25f : 0.03125f) : 0.015625f;
+  const bool small = __all_sync(mask, hb < kSmall);
+  const bool tiny = __all_sync(mask, hb < kTiny);
   // the common layout (r_one's SIMPLE), decided for the whole group
   constexpr bool YM = !IMAG && (F & F_REND) && (F & F_RSTART);
   const bool simple = __all_sync(mask, p2 == nullptr && (a.omega_pieces & 2) == 0 && (!YM || ymerge));
 #define SPGPE_R_POINTS(TIER, S)                                                                                      \
   r_points<T, LOGN, LOGE, F, TIER, S, K>(pu, pd, t, jo, y, tab, ty, p2, gh11, gh22, gh12, htau, xang, pieces, ymerge, \
                                          tm, sm, su, sd, nsum)
-  if constexpr (sizeof(T) == 8) {
-    if (simple)
-      SPGPE_R_POINTS(2, true);
-    else
-      SPGPE_R_POINTS(2, false);
-  } else if (simple) {
+  if (simple) {
     if (tiny)
       SPGPE_R_POINTS(0, true);
     else if (small)
