@@ -1864,9 +1864,9 @@ int observables_one(spgpe_ctx *c, void *p, double *out) {
   g.dy = c->dy;
   g.h = 0.5 * std::min(c->dx, c->dy);
   g.nb = (int)(std::sqrt(c->xmax * c->xmax + c->ymax * c->ymax) / g.h) + 2;
-  const int ni = c->ninst, sb = 128, npts = 4 * std::max(c->nx, c->ny);
-  // [ninst][nb] histogram, then R [ninst] and windings [ninst][2]
-  const size_t need = (size_t)ni * ((size_t)g.nb + 3);
+  const int ni = c->ninst, sb = std::min(128, c->ny), npts = 4 * std::max(c->nx, c->ny), nw = 2 * kWindBlocks;
+  // [ninst][nb] histogram, then R [ninst] and phase sums [ninst][2][kWindBlocks]
+  const size_t need = (size_t)ni * ((size_t)g.nb + 1 + nw);
   if (c->n_obs < need) {
     if (c->d_obs) cudaFree(c->d_obs);
     c->d_obs = nullptr;
@@ -1907,13 +1907,16 @@ int observables_one(spgpe_ctx *c, void *p, double *out) {
   }
   CK(c, cudaMemcpyAsync(dR, R.data(), R.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
   CK(c, launch_observables((int)c->es, p, g, ni, nullptr, sb, nullptr, dR, npts, dw, 1, c->st));
-  std::vector<double> w((size_t)ni * 2);
+  std::vector<double> w((size_t)ni * nw);
   CK(c, cudaMemcpyAsync(w.data(), dw, w.size() * sizeof(double), cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaStreamSynchronize(c->st));
   bool finite = true;
   for (int i = 0; i < ni; ++i) {
-    out[4 * (size_t)i + 1] = w[2 * (size_t)i];
-    out[4 * (size_t)i + 2] = w[2 * (size_t)i + 1];
+    for (int j = 0; j < 2; ++j) {
+      double s = 0.0;
+      for (int k = 0; k < kWindBlocks; ++k) s += w[(size_t)i * nw + (size_t)j * kWindBlocks + k];
+      out[4 * (size_t)i + 1 + j] = std::rint(s / kTwoPi);
+    }
     for (int k = 0; k < 4; ++k) finite = finite && std::isfinite(out[4 * (size_t)i + k]);
   }
   return finite ? SPGPE_OK : fail(c, SPGPE_ENONFINITE, "non-finite observable");

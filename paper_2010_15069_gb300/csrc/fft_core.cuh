@@ -25,6 +25,17 @@ struct alignas(2 * sizeof(T)) cx {
   T re, im;
 };
 
+// A float as a double, exactly, with integer instructions where it is a normal
+// number or zero (an FP64 conversion runs at the FP64 rate, which bounds the
+// FP64 sums over single-precision spinors).
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
+  if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)f;  // subnormal, infinite or NaN
+  const unsigned hi = a == 0u ? 0u : (a >> 3) + 0x38000000u;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
 template <class T> __device__ __forceinline__ T d_fma(T a, T b, T c) {
   if constexpr (sizeof(T) == 4) return fmaf(a, b, c); else return fma(a, b, c);
 }

@@ -776,6 +776,10 @@ __device__ __forceinline__ int kbin(int i, int n) { return i < n / 2 ? i : i - n
 
 // Real-space energy densities (trap, detuning, Raman, interaction, atom
 // numbers) in FP64, then the forward x-FFT of both components into scratch.
+// Bound by the FP64 units: a point takes 13 FP64 instructions with separable
+// potentials (the y pieces multiply a row's sums once; the x pieces of detuning
+// and Raman coupling only where they are present), all conversions are
+// integer work (widen).
 template <class T, int LOGN, int LOGE>
 __global__ void __launch_bounds__(2 * kRowMaxThreads) energy_row(const EnergyArgs a) {
   constexpr int N = 1 << LOGN, E = 1 << LOGE, TT = N / E;
@@ -797,29 +801,40 @@ __global__ void __launch_bounds__(2 * kRowMaxThreads) energy_row(const EnergyArg
   const double g11 = a.gpar[4 * inst], g22 = a.gpar[4 * inst + 1], g12 = a.gpar[4 * inst + 2];
 
   cx<T> v[2][E];
-  double acc6[6] = {0, 0, 0, 0, 0, 0};  // trap, detuning, Raman, interaction, N_up, N_dn
+  double su = 0, sd = 0, sv = 0, sde = 0, sc = 0, so = 0, suu = 0, sdd = 0, sud = 0;
 #pragma unroll
   for (int m = 0; m < E; ++m) {
     const int x = t + m * TT;
     v[0][m] = up[x];
     v[1][m] = dn[x];
+    const double ur = widen(v[0][m].re), ui = widen(v[0][m].im), dr = widen(v[1][m].re), di = widen(v[1][m].im);
+    const double ru = fma(ur, ur, ui * ui), rd = fma(dr, dr, di * di);
     const q4<T> px = rx[x];
-    double V = double(px.x) + double(ry.x), de = double(px.y) + double(ry.y), Om = double(px.z) + double(ry.z);
+    su += ru;
+    sd += rd;
+    sv = fma(widen(px.x), ru + rd, sv);
+    if (px.y != T(0)) sde = fma(widen(px.y), ru - rd, sde);
+    sc = fma(ur, dr, sc);
+    sc = fma(ui, di, sc);
+    if (px.z != T(0)) so = fma(widen(px.z), fma(ur, dr, ui * di), so);
+    suu = fma(ru, ru, suu);
+    sdd = fma(rd, rd, sdd);
+    sud = fma(ru, rd, sud);
     if (p2) {
       const q4<T> q = p2[(long)y * N + x];
-      V += 0.5 * (double(q.x) + double(q.y));
-      de += double(q.x) - double(q.y);
-      Om += double(q.z);
+      const double qu = widen(q.x), qd = widen(q.y);
+      sv = fma(0.5 * (qu + qd), ru + rd, sv);
+      sde = fma(qu - qd, ru - rd, sde);
+      so = fma(widen(q.z), fma(ur, dr, ui * di), so);
     }
-    const double ur = v[0][m].re, ui = v[0][m].im, dr = v[1][m].re, di = v[1][m].im;
-    const double ru = ur * ur + ui * ui, rd = dr * dr + di * di;
-    acc6[0] += V * (ru + rd);
-    acc6[1] += 0.5 * de * (ru - rd);
-    acc6[2] += Om * (ur * dr + ui * di);
-    acc6[3] += 0.5 * g11 * ru * ru + 0.5 * g22 * rd * rd + g12 * ru * rd;
-    acc6[4] += ru;
-    acc6[5] += rd;
   }
+  // trap, detuning, Raman, interaction, N_up, N_dn
+  double acc6[6] = {fma(widen(ry.x), su + sd, sv),
+                    0.5 * fma(widen(ry.y), su - sd, sde),
+                    fma(widen(ry.z), sc, so),
+                    fma(0.5 * g11, suu, fma(0.5 * g22, sdd, g12 * sud)),
+                    su,
+                    sd};
   block_sum<6>(acc6);
   if (threadIdx.x == 0)
 #pragma unroll
@@ -833,47 +848,62 @@ __global__ void __launch_bounds__(2 * kRowMaxThreads) energy_row(const EnergyArg
 }
 
 // Forward y-FFT of the scratch columns and the kinetic sum
-// sum_k T_j(k) |psi_hat_j(k)|^2 with T_j = k^2/2 -+ kL kx, in FP64.
+// sum_k T_j(k) |psi_hat_j(k)|^2 with T_j = k^2/2 -+ kL kx, in FP64: per point the
+// squared magnitude, its sum and its sum with ky^2 / 2 (from a shared-memory
+// table), the column's kx part once at the end.
 template <class T, int LOGN, int LOGE>
 __global__ void __launch_bounds__(512) energy_col(const EnergyArgs a) {
   constexpr int N = 1 << LOGN, E = 1 << LOGE, TT = N / E;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ double ky2[N];
   const int C = a.C;
   const int c = threadIdx.x % C, t = threadIdx.x / C;
   const int comp = blockIdx.y, inst = blockIdx.z;
   const int ix = blockIdx.x * C + c;
   const cx<T> *col = reinterpret_cast<const cx<T> *>(a.scratch) + ((long)inst * 2 + comp) * (long)N * a.nx + ix;
   const ColAcc<T> acc{reinterpret_cast<cx<T> *>(smem_raw), C, c};
+  for (int k = threadIdx.x; k < N; k += blockDim.x) {
+    const double ky = a.dky * kbin(k, N);
+    ky2[k] = 0.5 * ky * ky;
+  }
   cx<T> v[1][E];
 #pragma unroll
   for (int m = 0; m < E; ++m) v[0][m] = col[(long)(t + m * TT) * a.nx];
+  __syncthreads();
   block_fft<LOGN, LOGE, -1, 1>(v, t, a.twy, acc);
   const double kL = a.gpar[4 * inst + 3];
   const double kx = a.dkx * kbin(ix, a.nx);
   const double shift = (comp == 0 ? -kL : kL) * kx;
-  double s[1] = {0.0};
+  double sp = 0.0, sk = 0.0;
 #pragma unroll
   for (int m = 0; m < E; ++m) {
-    const double ky = a.dky * kbin(t + m * TT, N);
-    const double re = v[0][m].re, im = v[0][m].im;
-    s[0] += (0.5 * (kx * kx + ky * ky) + shift) * (re * re + im * im);
+    const double re = widen(v[0][m].re), im = widen(v[0][m].im);
+    const double p = fma(re, re, im * im);
+    sp += p;
+    sk = fma(ky2[t + m * TT], p, sk);
   }
+  double s[1] = {fma(0.5 * kx * kx + shift, sp, sk)};
   block_sum<1>(s);
   if (threadIdx.x == 0) a.partials[((long)inst * 2 + comp) * gridDim.x + blockIdx.x] = s[0];
 }
 
 // ---------------------------------------------------- generic reductions
 
+// (Two FP64 instructions per point and component: what bounds it.)
 template <class T>
 __global__ void __launch_bounds__(256) norm_kernel(const cx<T> *__restrict__ psi, long plane,
                                                    double *__restrict__ partials) {
   const int inst = blockIdx.y;
   const cx<T> *u = psi + (long)inst * 2 * plane, *d = u + plane;
   double s[2] = {0.0, 0.0};
+#pragma unroll 4
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < plane; i += (long)gridDim.x * blockDim.x) {
     const cx<T> a = u[i], b = d[i];
-    s[0] += double(a.re) * a.re + double(a.im) * a.im;
-    s[1] += double(b.re) * b.re + double(b.im) * b.im;
+    const double ar = widen(a.re), ai = widen(a.im), br = widen(b.re), bi = widen(b.im);
+    s[0] = fma(ar, ar, s[0]);
+    s[0] = fma(ai, ai, s[0]);
+    s[1] = fma(br, br, s[1]);
+    s[1] = fma(bi, bi, s[1]);
   }
   block_sum<2>(s);
   if (threadIdx.x == 0) {
@@ -888,11 +918,14 @@ __global__ void __launch_bounds__(256) residual_kernel(const cx<T> *__restrict__
   const int inst = blockIdx.y;
   const long base = (long)inst * 2 * plane;
   double s[2] = {0.0, 0.0};
+#pragma unroll 4
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < 2 * plane; i += (long)gridDim.x * blockDim.x) {
     const cx<T> a = psi[base + i], b = prev[base + i];
-    const double dr = double(a.re) - b.re, di = double(a.im) - b.im;
-    s[0] += dr * dr + di * di;
-    s[1] += double(b.re) * b.re + double(b.im) * b.im;
+    const double br = widen(b.re), bi = widen(b.im), dr = widen(a.re) - br, di = widen(a.im) - bi;
+    s[0] = fma(dr, dr, s[0]);
+    s[0] = fma(di, di, s[0]);
+    s[1] = fma(br, br, s[1]);
+    s[1] = fma(bi, bi, s[1]);
   }
   block_sum<2>(s);
   if (threadIdx.x == 0) {

@@ -1,10 +1,10 @@
 // Observables of the spin-Hall ground states (Sec. 6) and the annealing noise
 // of the ground-state protocol, both precisions.
 //
-//  * obs_sums: FP64 sums rho_up rho_dn, rho_up^2, rho_dn^2 and rho_up + rho_dn
-//    per instance (the phase-separation parameter of Eq. 14 and the total).
-//  * radial_hist: atom number in radial bins of width h about the trap centre
-//    (the contour of Eq. 15 encloses 99 % of it).
+//  * sums_and_hist: FP64 sums rho_up rho_dn, rho_up^2, rho_dn^2 and rho_up +
+//    rho_dn per instance (the phase-separation parameter of Eq. 14 and the
+//    total), and the atom number in radial bins of width h about the trap
+//    centre (the contour of Eq. 15 encloses 99 % of it), in one read of psi.
 //  * winding: phase steps of psi_j (bilinearly interpolated) around the circle
 //    of radius R99, summed in FP64 (Eq. 15 winding numbers).
 //  * add_noise: psi += sigma xi, xi complex standard normal from a
@@ -41,30 +41,15 @@ template <int K> __device__ __forceinline__ void obs_block_sum(double (&v)[K]) {
   __syncthreads();
 }
 
+// One block per (row group, instance): the FP64 sums of its rows into
+// partials[inst][block][4], and a shared-memory histogram of nb bins merged into
+// hist[inst][nb] (zeroed by the caller).  The radius over h is taken in
+// float32 first; within 1/128 of a whole number (beyond its rounding for every
+// grid: at most 4096 points, 8192 bins) the FP64 value decides, so the bins are
+// those of FP64 throughout without a square root and a division per point.
 template <class T>
-__global__ void __launch_bounds__(256) obs_sums(const cx<T> *__restrict__ psi, long plane, double *partials) {
-  const int inst = blockIdx.y;
-  const cx<T> *u = psi + (long)inst * 2 * plane, *d = u + plane;
-  double s[4] = {0.0, 0.0, 0.0, 0.0};
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < plane; i += (long)gridDim.x * blockDim.x) {
-    const cx<T> a = u[i], b = d[i];
-    const double ru = double(a.re) * a.re + double(a.im) * a.im;
-    const double rd = double(b.re) * b.re + double(b.im) * b.im;
-    s[0] += ru * rd;
-    s[1] += ru * ru;
-    s[2] += rd * rd;
-    s[3] += ru + rd;
-  }
-  obs_block_sum<4>(s);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 4; ++k) partials[((long)inst * gridDim.x + blockIdx.x) * 4 + k] = s[k];
-}
-
-// One block per (row group, instance): a shared-memory histogram of nb bins,
-// merged into hist[inst][nb] (zeroed by the caller).
-template <class T>
-__global__ void __launch_bounds__(256) radial_hist(const cx<T> *__restrict__ psi, ObsGeom g, int rows_per_block,
-                                                   double *hist) {
+__global__ void __launch_bounds__(256) sums_and_hist(const cx<T> *__restrict__ psi, ObsGeom g, int rows_per_block,
+                                                     double *partials, double *hist) {
   extern __shared__ double sh[];
   const int inst = blockIdx.y;
   for (int b = threadIdx.x; b < g.nb; b += blockDim.x) sh[b] = 0.0;
@@ -73,13 +58,31 @@ __global__ void __launch_bounds__(256) radial_hist(const cx<T> *__restrict__ psi
   const cx<T> *u = psi + (long)inst * 2 * plane, *d = u + plane;
   const int y0 = blockIdx.x * rows_per_block;
   const int y1 = min(g.ny, y0 + rows_per_block);
+  const float dxf = (float)(g.dx / g.h), dyf = (float)(g.dy / g.h);
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  const int lx = __ffs(g.nx) - 1;  // nx is a power of two
   for (long i = (long)y0 * g.nx + threadIdx.x; i < (long)y1 * g.nx; i += blockDim.x) {
-    const int iy = (int)(i / g.nx), ix = (int)(i - (long)iy * g.nx);
-    const double x = -g.xmax + ix * g.dx, y = -g.ymax + iy * g.dy;
-    const int bin = min(g.nb - 1, (int)(sqrt(x * x + y * y) / g.h));
+    const int iy = (int)(i >> lx), ix = (int)(i & (g.nx - 1));
     const cx<T> a = u[i], b = d[i];
-    atomicAdd(&sh[bin], double(a.re) * a.re + double(a.im) * a.im + double(b.re) * b.re + double(b.im) * b.im);
+    const double ar = widen(a.re), ai = widen(a.im), br = widen(b.re), bi = widen(b.im);
+    const double ru = fma(ar, ar, ai * ai), rd = fma(br, br, bi * bi), r = ru + rd;
+    s[0] = fma(ru, rd, s[0]);
+    s[1] = fma(ru, ru, s[1]);
+    s[2] = fma(rd, rd, s[2]);
+    s[3] += r;
+    // -xmax + ix dx = (ix - nx / 2) dx
+    const float xf = (float)(ix - g.nx / 2) * dxf, yf = (float)(iy - g.ny / 2) * dyf;
+    const float rf = sqrtf(fmaf(xf, xf, yf * yf)), ff = rf - floorf(rf);
+    int bin = (int)rf;
+    if (ff < 0.0078125f || ff > 0.9921875f) {
+      const double x = -g.xmax + ix * g.dx, y = -g.ymax + iy * g.dy;
+      bin = (int)(sqrt(x * x + y * y) / g.h);
+    }
+    if (r != 0.0) atomicAdd(&sh[min(g.nb - 1, bin)], r);
   }
+  obs_block_sum<4>(s);
+  if (threadIdx.x == 0)
+    for (int k = 0; k < 4; ++k) partials[((long)inst * gridDim.x + blockIdx.x) * 4 + k] = s[k];
   __syncthreads();
   for (int b = threadIdx.x; b < g.nb; b += blockDim.x)
     if (sh[b] != 0.0) atomicAdd(&hist[(long)inst * g.nb + b], sh[b]);
@@ -99,28 +102,42 @@ template <class T> __device__ __forceinline__ double phase_at(const cx<T> *f, co
   return atan2(im, re);
 }
 
-// One block per (component, instance): sum of the wrapped phase steps around
-// the circle of radius R[inst] with npts points; out[inst][comp] = n.
+// Sum of the wrapped phase steps around the circle of radius R[inst] with npts
+// points, over the block's share of them (one of kWindBlocks per component and
+// instance): out[inst][comp][block], for the host to add and round.  Each
+// point's phase is taken once and its neighbour's read from shared memory (a
+// phase is about a hundred FP64 instructions); with one block per component and
+// every phase taken twice, 16 instances of 512^2 took 144 us on 32 SMs.
+constexpr int kWindThreads = 256;
 template <class T>
-__global__ void __launch_bounds__(256) winding(const cx<T> *__restrict__ psi, ObsGeom g, const double *R, int npts,
-                                               double *out) {
-  const int comp = blockIdx.x, inst = blockIdx.y;
+__global__ void __launch_bounds__(kWindThreads) winding(const cx<T> *__restrict__ psi, ObsGeom g, const double *R,
+                                                        int npts, double *out) {
+  __shared__ double ph[kWindThreads + 1];
+  const int comp = blockIdx.y, inst = blockIdx.z;
   const long plane = (long)g.nx * g.ny;
   const cx<T> *f = psi + ((long)inst * 2 + comp) * plane;
   const double r = R[inst];
+  const double pi = 3.14159265358979323846;
+  const int per = (npts + gridDim.x - 1) / gridDim.x, k1 = min(npts, (int)(blockIdx.x + 1) * per);
   double s[1] = {0.0};
-  for (int k = threadIdx.x; k < npts; k += blockDim.x) {
-    double s0, c0, s1, c1;
-    sincospi(2.0 * k / npts, &s0, &c0);
-    sincospi(2.0 * ((k + 1) % npts) / npts, &s1, &c1);
-    double dph = phase_at(f, g, r * c1, r * s1) - phase_at(f, g, r * c0, r * s0);
-    const double pi = 3.14159265358979323846;
-    while (dph > pi) dph -= 2.0 * pi;
-    while (dph <= -pi) dph += 2.0 * pi;
-    s[0] += dph;
+  for (int k0 = blockIdx.x * per; k0 < k1; k0 += kWindThreads) {
+    const int n = min(kWindThreads, k1 - k0);  // steps k0 .. k0 + n - 1, phases k0 .. k0 + n
+    for (int j = threadIdx.x; j <= n; j += kWindThreads) {
+      double sn, cs;
+      sincospi(2.0 * ((k0 + j) % npts) / npts, &sn, &cs);
+      ph[j] = phase_at(f, g, r * cs, r * sn);
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < n) {
+      double dph = ph[threadIdx.x + 1] - ph[threadIdx.x];
+      while (dph > pi) dph -= 2.0 * pi;
+      while (dph <= -pi) dph += 2.0 * pi;
+      s[0] += dph;
+    }
+    __syncthreads();
   }
   obs_block_sum<1>(s);
-  if (threadIdx.x == 0) out[(long)inst * 2 + comp] = rint(s[0] / (2.0 * 3.14159265358979323846));
+  if (threadIdx.x == 0) out[((long)inst * 2 + comp) * gridDim.x + blockIdx.x] = s[0];
 }
 
 // SplitMix64 (Steele, Lea & Flood, OOPSLA 2014) as a counter-based generator:
@@ -159,16 +176,15 @@ template <class T> cudaError_t obs_launch(const void *psi, const ObsGeom &g, int
                                           int phase, cudaStream_t st) {
   const cx<T> *p = reinterpret_cast<const cx<T> *>(psi);
   if (phase == 0) {
-    obs_sums<T><<<dim3(sum_blocks, ninst), 256, 0, st>>>(p, (long)g.nx * g.ny, partials);
-    const int rpb = (g.ny + 63) / 64;  // 64 row groups per instance
+    const int rpb = (g.ny + sum_blocks - 1) / sum_blocks;
     const size_t sm = (size_t)g.nb * sizeof(double);
     if (sm > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(radial_hist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      const cudaError_t e = cudaFuncSetAttribute(sums_and_hist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    radial_hist<T><<<dim3((g.ny + rpb - 1) / rpb, ninst), 256, sm, st>>>(p, g, rpb, hist);
+    sums_and_hist<T><<<dim3(sum_blocks, ninst), 256, sm, st>>>(p, g, rpb, partials, hist);
   } else {
-    winding<T><<<dim3(2, ninst), 256, 0, st>>>(p, g, R, npts, wind);
+    winding<T><<<dim3(kWindBlocks, 2, ninst), kWindThreads, 0, st>>>(p, g, R, npts, wind);
   }
   return cudaGetLastError();
 }
