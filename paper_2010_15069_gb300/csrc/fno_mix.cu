@@ -15,7 +15,9 @@
 // 132 us transposed, 74 us for the gradient, then 475 us of Adam over the
 // whole parameter vector and a cleared gradient): a training step of the
 // full-size network at 256^2 8.8 -> 7.7 ms, its inference at 512^2 8.1 -> 7.7
-// ms.
+// ms.  The gradient with its Adam step moves 436 MB (64 us at the copy rate):
+// 140 us with one block for all rows of four modes, 117 us with four rows'
+// loads ahead of their use, 92 us with 16 rows per block.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -150,25 +152,29 @@ __global__ void __launch_bounds__(32 * kModes) mix(const __nv_bfloat162 *__restr
 // or (g null) applied at once as the weights' Adam step, so that the
 // gradient never goes through memory: w, m, v read and written, the bfloat16
 // weights written, 26 bytes per parameter.  One warp per mode, four modes per
-// block; a lane owns adjacent columns c and walks the rows o.
-constexpr int kGradModes = 4;
+// block and kGradRows of the rows o (so that a layer has many more blocks
+// than there is room for at once); a lane owns adjacent columns c and walks the rows, four at a time.
+constexpr int kGradModes = 4, kGradRows = 16;
 
 template <int W, int BG, bool ADAM>
 __global__ void __launch_bounds__(32 * kGradModes) mix_grad(const float2 *__restrict__ d, const float2 *__restrict__ v,
-                                                            long modes, int batch, float2 *g, float2 *w, float2 *mo,
-                                                            float2 *ve, __nv_bfloat162 *wb, AdamRates ar) {
+                                                            long modes, int batch, float2 *__restrict__ g,
+                                                            float2 *__restrict__ w, float2 *__restrict__ mo,
+                                                            float2 *__restrict__ ve, __nv_bfloat162 *__restrict__ wb,
+                                                            AdamRates ar) {
   constexpr int NC = W / 32;
   constexpr int ST = W * BG + 2;
   __shared__ __align__(16) float2 s[kGradModes * ST];
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int row0 = blockIdx.y * kGradRows, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const long m0 = (long)blockIdx.x * kGradModes, m = m0 + wp;
-  auto load = [&](const float2 *__restrict__ src) {
-    for (int e = threadIdx.x; e < BG * W * kGradModes; e += blockDim.x) {
-      const int i = e & (kGradModes - 1), bc = e / kGradModes;
-      s[i * ST + bc] = bc / W < batch ? src[(long)bc * modes + m0 + i] : make_float2(0.f, 0.f);
+  // [sample][nc channels from c0]
+  auto load = [&](const float2 *__restrict__ src, int c0, int nc) {
+    for (int e = threadIdx.x; e < BG * nc * kGradModes; e += blockDim.x) {
+      const int i = e & (kGradModes - 1), bc = e / kGradModes, b = bc / nc;
+      s[i * ST + bc] = b < batch ? src[((long)b * W + c0 + bc - b * nc) * modes + m0 + i] : make_float2(0.f, 0.f);
     }
   };
-  load(v);
+  load(v, 0, W);
   __syncthreads();
   const float2 *sm = s + wp * ST;
   float2 vc[NC][BG];  // the lane's columns of v
@@ -177,44 +183,53 @@ __global__ void __launch_bounds__(32 * kGradModes) mix_grad(const float2 *__rest
 #pragma unroll
     for (int b = 0; b < BG; ++b) vc[i][b] = sm[b * W + NC * lane + i];
   __syncthreads();
-  load(d);
+  load(d, row0, kGradRows);
   __syncthreads();
-#pragma unroll 4
-  for (int o = 0; o < W; ++o) {
-    const long p = (m * W + o) * W + NC * lane;
-    using V = Cols<NC>;
-    V wv, mv, vv;
+  // four rows' weights and moments are on their way before the first is needed
+  constexpr int G = ADAM ? 4 : 1;
+  using V = Cols<NC>;
+#pragma unroll 1
+  for (int o0 = 0; o0 < kGradRows; o0 += G) {
+    const long p0 = (m * W + row0 + o0) * W + NC * lane;
+    V wv[G], mv[G], vv[G];
     if constexpr (ADAM) {
-      wv = *reinterpret_cast<const V *>(w + p);
-      mv = *reinterpret_cast<const V *>(mo + p);
-      vv = *reinterpret_cast<const V *>(ve + p);
-    }
-    V gr;
 #pragma unroll
-    for (int i = 0; i < NC; ++i) gr.e[i] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int b = 0; b < BG; ++b) {
-      const float2 dv = sm[b * W + o];
-#pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        gr.e[i].x = fmaf(dv.x, vc[i][b].x, fmaf(dv.y, vc[i][b].y, gr.e[i].x));
-        gr.e[i].y = fmaf(dv.y, vc[i][b].x, fmaf(-dv.x, vc[i][b].y, gr.e[i].y));
+      for (int q = 0; q < G; ++q) {
+        wv[q] = *reinterpret_cast<const V *>(w + p0 + q * W);
+        mv[q] = *reinterpret_cast<const V *>(mo + p0 + q * W);
+        vv[q] = *reinterpret_cast<const V *>(ve + p0 + q * W);
       }
     }
-    if constexpr (ADAM) {
-      ColsB<NC> r;
 #pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        adam_one(wv.e[i].x, mv.e[i].x, vv.e[i].x, gr.e[i].x, ar);
-        adam_one(wv.e[i].y, mv.e[i].y, vv.e[i].y, gr.e[i].y, ar);
-        r.e[i] = __floats2bfloat162_rn(wv.e[i].x, wv.e[i].y);
+    for (int q = 0; q < G; ++q) {
+      const long p = p0 + q * W;
+      V gr;
+#pragma unroll
+      for (int i = 0; i < NC; ++i) gr.e[i] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int b = 0; b < BG; ++b) {
+        const float2 dv = sm[b * kGradRows + o0 + q];
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          gr.e[i].x = fmaf(dv.x, vc[i][b].x, fmaf(dv.y, vc[i][b].y, gr.e[i].x));
+          gr.e[i].y = fmaf(dv.y, vc[i][b].x, fmaf(-dv.x, vc[i][b].y, gr.e[i].y));
+        }
       }
-      *reinterpret_cast<V *>(w + p) = wv;
-      *reinterpret_cast<V *>(mo + p) = mv;
-      *reinterpret_cast<V *>(ve + p) = vv;
-      *reinterpret_cast<ColsB<NC> *>(wb + p) = r;
-    } else {
-      *reinterpret_cast<V *>(g + p) = gr;
+      if constexpr (ADAM) {
+        ColsB<NC> r;
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          adam_one(wv[q].e[i].x, mv[q].e[i].x, vv[q].e[i].x, gr.e[i].x, ar);
+          adam_one(wv[q].e[i].y, mv[q].e[i].y, vv[q].e[i].y, gr.e[i].y, ar);
+          r.e[i] = __floats2bfloat162_rn(wv[q].e[i].x, wv[q].e[i].y);
+        }
+        *reinterpret_cast<V *>(w + p) = wv[q];
+        *reinterpret_cast<V *>(mo + p) = mv[q];
+        *reinterpret_cast<V *>(ve + p) = vv[q];
+        *reinterpret_cast<ColsB<NC> *>(wb + p) = r;
+      } else {
+        *reinterpret_cast<V *>(g + p) = gr;
+      }
     }
   }
 }
@@ -236,7 +251,7 @@ cudaError_t mix_w(const void *R, const float2 *in, float2 *out, long modes, int 
 template <int W, bool ADAM>
 cudaError_t grad_w(const float2 *d, const float2 *v, long modes, int batch, float *g, float *w, float *m, float *ve,
                    void *wb, const AdamRates &ar, cudaStream_t st) {
-  const unsigned grid = (unsigned)(modes / kGradModes);
+  const dim3 grid((unsigned)(modes / kGradModes), W / kGradRows);
   auto go = [&](auto kern) {
     kern<<<grid, 32 * kGradModes, 0, st>>>(d, v, modes, batch, reinterpret_cast<float2 *>(g),
                                            reinterpret_cast<float2 *>(w), reinterpret_cast<float2 *>(m),
