@@ -42,7 +42,7 @@ struct spgpe_fno {
   float2 *Ey = nullptr;
   uint16_t *tab[2] = {};  // tensor-core transforms' tables, by DftTable
   float *sin32 = nullptr;
-  float2 *EyT = nullptr;  // Ey by y: [y][j]
+  float4 *EyT = nullptr;  // Ey by y: [y][j], in the pairs dft_y multiplies with
   int sms = 0;
   // workspace for (ws_b, ws_n)
   int ws_b = 0, ws_n = 0;
@@ -137,10 +137,15 @@ int ensure_twiddles(spgpe_fno *f, int n) {
       if ((r = falloc(f, &f->tab[i], t.size()))) return r;
       FCK(f, cudaMemcpy(f->tab[i], t.data(), t.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
     }
-    std::vector<float> eyt(ey.size());
+    std::vector<float> eyt(ey.size() * 2);
     for (int j = 0; j < 2 * M; ++j)
-      for (int y = 0; y < n; ++y)
-        for (int c = 0; c < 2; ++c) eyt[((size_t)y * 2 * M + j) * 2 + c] = ey[((size_t)j * n + y) * 2 + c];
+      for (int y = 0; y < n; ++y) {
+        const float re = ey[((size_t)j * n + y) * 2], im = ey[((size_t)j * n + y) * 2 + 1];
+        float *o = &eyt[((size_t)y * 2 * M + j) * 4];
+        o[0] = o[1] = re;
+        o[2] = -im;
+        o[3] = im;
+      }
     if ((r = falloc(f, &f->EyT, (size_t)2 * M * n))) return r;
     FCK(f, cudaMemcpy(f->EyT, eyt.data(), eyt.size() * sizeof(float), cudaMemcpyHostToDevice));
     std::vector<float> s32((size_t)n);

@@ -21,8 +21,8 @@
 // shared-memory image, fetched by bulk copies.
 //
 // Measured on GB300 (256 images = batch 4 x 64 channels, 32 modes) against the
-// general products: at 256^2 along x 116 -> 53 us, along y 126 -> 44 us, inverse
-// along y 76 -> 14 us; at 512^2 442 -> 170, 126 -> 84 and 129 -> 24 us.  (On the
+// general products: at 256^2 along x 116 -> 53 us, along y 126 -> 42 us, inverse
+// along y 76 -> 14 us; at 512^2 442 -> 170, 126 -> 80 and 129 -> 24 us.  (On the
 // tensor cores, split like the inverse, the forward transforms took 32 and 13
 // us at 256^2 and came out nearer to the 64-bit result; weights trained for a
 // few steps then differ from those of the general path by that path's own
@@ -152,26 +152,30 @@ __global__ void __launch_bounds__(128, 3) dft_rows(const float *__restrict__ v, 
 
 // Along y: one image per 256 threads (or several small ones), 4 wavenumbers j x
 // 2 kx per thread, blocks of 32 y, the next y's operands in registers.  The
-// complex term a b is two packed fma: (-a.y, a.y) (b.y, b.x), then (a.x, a.x)
-// (b.x, b.y).
+// complex term a b is two packed fma, (-a.y, a.y) (b.y, b.x), then (a.x, a.x)
+// (b.x, b.y); the table holds the pairs (a.x, a.x, -a.y, a.y) ready, so that the
+// 16 packed fma of a y need no register shuffling but b's swap (44 -> 42 us at
+// 256^2, 84 -> 80 us at 512^2).
 constexpr int kYBlock = 32, kYThreads = 256;
 
-__global__ void __launch_bounds__(kYThreads, 2) dft_cols(const float2 *__restrict__ X1, const float2 *__restrict__ Et, int n,
+__global__ void __launch_bounds__(kYThreads, 2) dft_cols(const float2 *__restrict__ X1, const float4 *__restrict__ Et, int n,
                                                       int M, int images, int per_block, float2 *__restrict__ out) {
-  extern __shared__ __align__(16) float2 smem_c[];
+  extern __shared__ __align__(16) float4 smem_c[];
   const int J = 2 * M, jt = (J + 3) / 4, kt = M / 2, Jp = 4 * jt;  // (M is even) wavenumbers padded to whole thread tiles
-  float2 *se = smem_c, *sx = smem_c + 2 * kYBlock * Jp;            // [2][y][Jp], [2][image][y][M]
+  float4 *se = smem_c;                                             // [2][y][Jp]
+  float2 *sx = reinterpret_cast<float2 *>(smem_c + 2 * kYBlock * Jp);  // [2][image][y][M]
   const int tid = threadIdx.x, per = jt * kt;
   const int im = min(tid / per, per_block - 1), loc = tid % per, tj = loc / kt, tk = loc - tj * kt;
   const int img0 = blockIdx.x * per_block;
   const bool mine = tid < per * per_block && img0 + im < images;
   const int blocks = n / kYBlock;
   for (int e = tid; e < 2 * kYBlock * Jp; e += kYThreads)
-    if (e % Jp >= J) se[e] = make_float2(0.f, 0.f);
+    if (e % Jp >= J) se[e] = make_float4(0.f, 0.f, 0.f, 0.f);
   auto fetch = [&](int b) {
-    float2 *de = se + (b & 1) * kYBlock * Jp, *dx = sx + (b & 1) * per_block * kYBlock * M;
-    for (int e = tid; e < kYBlock * M; e += kYThreads) {  // two wavenumbers at a time (2M of them per y)
-      const int y = e / M, c = 2 * (e - y * M);
+    float4 *de = se + (b & 1) * kYBlock * Jp;
+    float2 *dx = sx + (b & 1) * per_block * kYBlock * M;
+    for (int e = tid; e < kYBlock * J; e += kYThreads) {
+      const int y = e / J, c = e - y * J;
       cp16(de + y * Jp + c, Et + (long)(b * kYBlock + y) * J + c);
     }
     const int h = kYBlock * M / 2;  // 16-byte pieces of an image's block, which is contiguous
@@ -196,26 +200,33 @@ __global__ void __launch_bounds__(kYThreads, 2) dft_cols(const float2 *__restric
       cp_wait<0>();
     }
     __syncthreads();
-    const float2 *pe = se + (b & 1) * kYBlock * Jp + 4 * tj;
+    const float4 *pe = se + (b & 1) * kYBlock * Jp + 4 * tj;
     const float2 *px = sx + ((b & 1) * per_block + im) * kYBlock * M + 2 * tk;
-    float4 e0 = *reinterpret_cast<const float4 *>(pe), e1 = *reinterpret_cast<const float4 *>(pe + 2);
-    float4 x0 = *reinterpret_cast<const float4 *>(px);
+    float4 en[4], xn = *reinterpret_cast<const float4 *>(px);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) en[j] = pe[j];
 #pragma unroll 8
     for (int y = 0; y < kYBlock; ++y) {
-      const float2 a[4] = {{e0.x, e0.y}, {e0.z, e0.w}, {e1.x, e1.y}, {e1.z, e1.w}};
-      const float2 x[2] = {{x0.x, x0.y}, {x0.z, x0.w}};
+      float4 a[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) a[j] = en[j];
+      const float4 x = xn;
       if (y + 1 < kYBlock) {
-        e0 = *reinterpret_cast<const float4 *>(pe + (y + 1) * Jp);
-        e1 = *reinterpret_cast<const float4 *>(pe + (y + 1) * Jp + 2);
-        x0 = *reinterpret_cast<const float4 *>(px + (y + 1) * M);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) en[j] = pe[(y + 1) * Jp + j];
+        xn = *reinterpret_cast<const float4 *>(px + (y + 1) * M);
+      }
+      const float2 x0 = make_float2(x.x, x.y), x1 = make_float2(x.z, x.w), s0 = make_float2(x.y, x.x),
+                   s1 = make_float2(x.w, x.z);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        acc[j][0] = __ffma2_rn(make_float2(a[j].z, a[j].w), s0, acc[j][0]);
+        acc[j][1] = __ffma2_rn(make_float2(a[j].z, a[j].w), s1, acc[j][1]);
       }
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const float2 s = make_float2(x[k].y, x[k].x);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[j][k] = __ffma2_rn(make_float2(-a[j].y, a[j].y), s, acc[j][k]);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[j][k] = __ffma2_rn(make_float2(a[j].x, a[j].x), x[k], acc[j][k]);
+      for (int j = 0; j < 4; ++j) {
+        acc[j][0] = __ffma2_rn(make_float2(a[j].x, a[j].y), x0, acc[j][0]);
+        acc[j][1] = __ffma2_rn(make_float2(a[j].x, a[j].y), x1, acc[j][1]);
       }
     }
     __syncthreads();  // the block's buffers are read: the block after next may go there
@@ -481,10 +492,10 @@ cudaError_t dft_x(const float *v, const float *E, bool adjoint, float *X1, int i
   }
 }
 
-cudaError_t dft_y(const float *X1, const float2 *Et, float2 *vh, int images, int n, int modes, cudaStream_t st) {
+cudaError_t dft_y(const float *X1, const float4 *Et, float2 *vh, int images, int n, int modes, cudaStream_t st) {
   const int jt = (2 * modes + 3) / 4, per_block = std::max(1, kYThreads / (jt * (modes / 2)));
-  const size_t smem = (size_t)2 * kYBlock * (4 * jt + per_block * modes) * sizeof(float2);
-  static size_t granted = 48 * 1024;
+  const size_t smem = (size_t)2 * kYBlock * (4 * jt * sizeof(float4) + per_block * modes * sizeof(float2));
+  static size_t granted = 0;
   const cudaError_t e = grant(dft_cols, smem, granted);
   if (e != cudaSuccess) return e;
   dft_cols<<<(unsigned)((images + per_block - 1) / per_block), kYThreads, smem, st>>>(reinterpret_cast<const float2 *>(X1), Et, n,

@@ -80,14 +80,14 @@ cudaError_t gemm_complex(const GemmC &g, cudaStream_t st);
 // kept modes kx < M, ky = -M .. M - 1 (M even, at most 32; n a multiple of 64;
 // `width` channels per sample, whose rows fill whole tiles of 128): along x
 // (E[x][2 k + part] = cos, -sin; adjoint: times g_k / n^2, g_0 = 1, g_k = 2) and
-// along y (Et[y][j] = exp(-2 pi i ky_j y / n)) in float32, the inverse along y
+// along y (Et[y][j] = (a.x, a.x, -a.y, a.y), a = exp(-2 pi i ky_j y / n)) in float32, the inverse along y
 // on the tensor cores (table: dft_table(InverseY) as it is; sin32[y] = sin(2 pi
 // 32 y / n)); flags receives a wait that ran out.
 enum class DftTable { InverseY, LayerX };
 bool dft_applies(int n, int modes, int width);
 std::vector<uint16_t> dft_table(DftTable which, int n, int modes);
 cudaError_t dft_x(const float *v, const float *E, bool adjoint, float *X1, int images, int n, int modes, cudaStream_t st);
-cudaError_t dft_y(const float *X1, const float2 *Et, float2 *vh, int images, int n, int modes, cudaStream_t st);
+cudaError_t dft_y(const float *X1, const float4 *Et, float2 *vh, int images, int n, int modes, cudaStream_t st);
 cudaError_t idft_y(const float2 *oh, const void *table, const float *sin32, float2 *G, int images, int n, int modes,
                    int *flags, cudaStream_t st);
 // The rest of a spectral layer in one pass (fno_layer.cu; W = 32 or 64 where
