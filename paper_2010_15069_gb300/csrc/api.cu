@@ -1864,7 +1864,7 @@ int observables_one(spgpe_ctx *c, void *p, double *out) {
   g.dy = c->dy;
   g.h = 0.5 * std::min(c->dx, c->dy);
   g.nb = (int)(std::sqrt(c->xmax * c->xmax + c->ymax * c->ymax) / g.h) + 2;
-  const int ni = c->ninst, sb = std::min(128, c->ny), npts = 4 * std::max(c->nx, c->ny), nw = 2 * kWindBlocks;
+  const int ni = c->ninst, sb = std::min(128, c->ny / 2), npts = 4 * std::max(c->nx, c->ny), nw = 2 * kWindBlocks;
   // [ninst][nb] histogram, then R [ninst] and phase sums [ninst][2][kWindBlocks]
   const size_t need = (size_t)ni * ((size_t)g.nb + 1 + nw);
   if (c->n_obs < need) {

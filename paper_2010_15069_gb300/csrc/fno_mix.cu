@@ -153,7 +153,8 @@ __global__ void __launch_bounds__(32 * kModes) mix(const __nv_bfloat162 *__restr
 // gradient never goes through memory: w, m, v read and written, the bfloat16
 // weights written, 26 bytes per parameter.  One warp per mode, four modes per
 // block and kGradRows of the rows o (so that a layer has many more blocks
-// than there is room for at once); a lane owns adjacent columns c and walks the rows, four at a time.
+// than there is room for at once); a lane owns adjacent columns c and walks the
+// rows, four at a time.
 constexpr int kGradModes = 4, kGradRows = 16;
 
 template <int W, int BG, bool ADAM>

@@ -43,10 +43,17 @@ template <int K> __device__ __forceinline__ void obs_block_sum(double (&v)[K]) {
 
 // One block per (row group, instance): the FP64 sums of its rows into
 // partials[inst][block][4], and a shared-memory histogram of nb bins merged into
-// hist[inst][nb] (zeroed by the caller).  The radius over h is taken in
-// float32 first; within 1/128 of a whole number (beyond its rounding for every
-// grid: at most 4096 points, 8192 bins) the FP64 value decides, so the bins are
-// those of FP64 throughout without a square root and a division per point.
+// hist[inst][nb] (zeroed by the caller).  What bounds it is the FP64 units, so
+// a bin costs no FP64 root and division but where it must: the radius over h is
+// taken in float32, and only within nb 2^-21 of a whole number (twice its
+// rounding) does each point's FP64 value decide; the bins are those of FP64
+// throughout.  A thread takes a point with its mirror images (columns c and nx -
+// c, rows r and ny - r; those without one, 0 and n / 2, go together) and adds the
+// four densities, which lie at one radius, as one; a warp adds up its runs of
+// equal bins before their first lane touches the histogram (FP64 additions in
+// shared memory are compare-and-swap loops).  Measured on GB300, 16 instances
+// of 512^2 in complex64: 294 us with an addition per point and FP64 radii, 251 us
+// with FP64 within 1/128 of an edge, 207 us as it is.
 template <class T>
 __global__ void __launch_bounds__(256) sums_and_hist(const cx<T> *__restrict__ psi, ObsGeom g, int rows_per_block,
                                                      double *partials, double *hist) {
@@ -56,29 +63,59 @@ __global__ void __launch_bounds__(256) sums_and_hist(const cx<T> *__restrict__ p
   __syncthreads();
   const long plane = (long)g.nx * g.ny;
   const cx<T> *u = psi + (long)inst * 2 * plane, *d = u + plane;
-  const int y0 = blockIdx.x * rows_per_block;
-  const int y1 = min(g.ny, y0 + rows_per_block);
-  const float dxf = (float)(g.dx / g.h), dyf = (float)(g.dy / g.h);
+  const int hx = g.nx / 2, hy = g.ny / 2, lx = __ffs(hx) - 1;  // nx is a power of two
+  const int r0 = blockIdx.x * rows_per_block, r1 = min(hy, r0 + rows_per_block);
+  const float dxf = (float)(g.dx / g.h), dyf = (float)(g.dy / g.h), edge = 0x1p-21f * g.nb;
   double s[4] = {0.0, 0.0, 0.0, 0.0};
-  const int lx = __ffs(g.nx) - 1;  // nx is a power of two
-  for (long i = (long)y0 * g.nx + threadIdx.x; i < (long)y1 * g.nx; i += blockDim.x) {
-    const int iy = (int)(i >> lx), ix = (int)(i & (g.nx - 1));
-    const cx<T> a = u[i], b = d[i];
-    const double ar = widen(a.re), ai = widen(a.im), br = widen(b.re), bi = widen(b.im);
-    const double ru = fma(ar, ar, ai * ai), rd = fma(br, br, bi * bi), r = ru + rd;
-    s[0] = fma(ru, rd, s[0]);
-    s[1] = fma(ru, ru, s[1]);
-    s[2] = fma(rd, rd, s[2]);
-    s[3] += r;
-    // -xmax + ix dx = (ix - nx / 2) dx
-    const float xf = (float)(ix - g.nx / 2) * dxf, yf = (float)(iy - g.ny / 2) * dyf;
-    const float rf = sqrtf(fmaf(xf, xf, yf * yf)), ff = rf - floorf(rf);
-    int bin = (int)rf;
-    if (ff < 0.0078125f || ff > 0.9921875f) {
-      const double x = -g.xmax + ix * g.dx, y = -g.ymax + iy * g.dy;
-      bin = (int)(sqrt(x * x + y * y) / g.h);
+  const int lane = threadIdx.x & 31, end = r1 << lx;
+  for (int base = r0 << lx; base < end; base += blockDim.x) {  // whole warps stay together
+    const int i = base + (int)threadIdx.x;
+    int bin = -1 - lane;  // equal to no neighbour's
+    double sum = 0.0;
+    if (i < end) {
+      const int row = i >> lx, col = i & (hx - 1);
+      const int iy[2] = {row, row == 0 ? hy : g.ny - row}, ix[2] = {col, col == 0 ? hx : g.nx - col};
+      cx<T> a[4], b[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const long p = (long)iy[q >> 1] * g.nx + ix[q & 1];
+        a[q] = u[p];
+        b[q] = d[p];
+      }
+      double r[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double ar = widen(a[q].re), ai = widen(a[q].im), br = widen(b[q].re), bi = widen(b[q].im);
+        const double ru = fma(ar, ar, ai * ai), rd = fma(br, br, bi * bi);
+        r[q] = ru + rd;
+        s[0] = fma(ru, rd, s[0]);
+        s[1] = fma(ru, ru, s[1]);
+        s[2] = fma(rd, rd, s[2]);
+      }
+      sum = (r[0] + r[1]) + (r[2] + r[3]);
+      s[3] += sum;
+      // -xmax + ix dx = (ix - nx / 2) dx
+      const float xf = (float)(col - hx) * dxf, yf = (float)(row - hy) * dyf;
+      const float rf = sqrtf(fmaf(xf, xf, yf * yf)), off = fabsf(rf - rintf(rf));
+      if (row != 0 && col != 0 && off >= edge) {
+        bin = min(g.nb - 1, (int)rf);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const double x = -g.xmax + ix[q & 1] * g.dx, y = -g.ymax + iy[q >> 1] * g.dy;
+          if (r[q] != 0.0) atomicAdd(&sh[min(g.nb - 1, (int)(sqrt(x * x + y * y) / g.h))], r[q]);
+        }
+      }
     }
-    if (r != 0.0) atomicAdd(&sh[min(g.nb - 1, bin)], r);
+    const int before = __shfl_up_sync(0xffffffffu, bin, 1);
+    const bool first = lane == 0 || bin != before;
+    const unsigned heads = __ballot_sync(0xffffffffu, first), later = lane == 31 ? 0u : heads >> (lane + 1);
+    const int stop = later ? lane + __ffs(later) : 32;  // one past the lane's run
+    for (int k = 1; __any_sync(0xffffffffu, lane + k < stop); k <<= 1) {
+      const double t = __shfl_down_sync(0xffffffffu, sum, k);
+      if (lane + k < stop) sum += t;
+    }
+    if (first && bin >= 0 && sum != 0.0) atomicAdd(&sh[bin], sum);
   }
   obs_block_sum<4>(s);
   if (threadIdx.x == 0)
@@ -176,7 +213,7 @@ template <class T> cudaError_t obs_launch(const void *psi, const ObsGeom &g, int
                                           int phase, cudaStream_t st) {
   const cx<T> *p = reinterpret_cast<const cx<T> *>(psi);
   if (phase == 0) {
-    const int rpb = (g.ny + sum_blocks - 1) / sum_blocks;
+    const int rpb = (g.ny / 2 + sum_blocks - 1) / sum_blocks;  // pairs of mirrored rows
     const size_t sm = (size_t)g.nb * sizeof(double);
     if (sm > 48 * 1024) {
       const cudaError_t e = cudaFuncSetAttribute(sums_and_hist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
