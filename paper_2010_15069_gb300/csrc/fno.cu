@@ -179,13 +179,7 @@ int ensure_workspace(spgpe_fno *f, int B, int n) {
   for (int l = 0; l < f->L; ++l)
     if ((r = falloc(f, &f->us[l], act)) || (r = falloc(f, &f->vh[l], spec)) || (r = falloc(f, &f->dohs[l], spec)))
       return r;
-  // split-K partials of the weight gradients: batch x splits x (largest weight)
-  const int splits = (int)std::max<size_t>(1, P / 1024);
-  size_t wmax = std::max<size_t>((size_t)f->W * f->cin, (size_t)f->W * f->W);
-  wmax = std::max(wmax, std::max((size_t)f->H * f->W, (size_t)f->cout * f->H));
-  // (of the general path; of the tensor-core weight gradients, a weight and a bias; of the projection)
-  f->part_n = std::max(std::max((size_t)B * splits * wmax, (size_t)2 * f->sms * (wmax + std::max(f->W, f->H))),
-                       (size_t)f->sms * (size_t)project_partials(f->H, f->cout));
+  f->part_n = partial_floats(f->cin, f->cout, f->W, f->H, B, (long)P, f->sms);
   if ((r = falloc(f, &f->X1, rows * 2)) || (r = falloc(f, &f->hp, hid)) || (r = falloc(f, &f->h, hid)) ||
       (r = falloc(f, &f->dh, hid)) || (r = falloc(f, &f->dv, act)) || (r = falloc(f, &f->dv2, act)) ||
       (r = falloc(f, &f->dout, (size_t)B * f->cout * P)) || (r = falloc(f, &f->oh, spec)) ||
@@ -252,6 +246,11 @@ cudaError_t greal(const spgpe_fno *f, GemmR g, cudaStream_t st) {
   return gemm_real(g, st);
 }
 
+// Room for the partial sums of a gradient, before their kernel is launched.
+int check_partials(spgpe_fno *f, size_t floats) {
+  return floats <= f->part_n ? SPGPE_OK : ffail(f, SPGPE_EINVAL, "partial sums of a gradient exceed their workspace");
+}
+
 // Report (and clear) an error recorded on the device; after a synchronisation.
 int read_flags(spgpe_fno *f) {
   int h = 0;
@@ -271,12 +270,14 @@ int wgrad(spgpe_fno *f, int M, int N, long P, int B, const float *A, long sAb, c
   if (f->tensor_cores && f->sms > 0 && weight_grad_applies(wg)) {
     const int parts = weight_grad_parts(B, P, f->sms);
     const long n = (long)M * N, stride = n + (bias ? M : 0);
+    if (const int r = check_partials(f, (size_t)parts * stride)) return r;
     FCK(f, weight_grad(wg, f->sms, f->st));
     FCK(f, sum_parts(f->part, stride, parts, n, grad, f->st));
     if (bias) FCK(f, sum_parts(f->part + n, stride, parts, M, bias, f->st));
     return SPGPE_OK;
   }
-  const int splits = (int)std::max<long>(1, P / 1024);
+  const int splits = general_splits(P);
+  if (const int r = check_partials(f, (size_t)B * splits * M * N)) return r;
   GemmR g = rg(M, N, (int)P, A, false, P, 1, Bm, 1, P, f->part, N, 1);
   g.batch = B;
   g.sAb = sAb;
@@ -428,9 +429,10 @@ int gradient(spgpe_fno *f, const float *a, const float *target, int B, int n, fl
   // output layer
   GemmR g;
   if (use_head(f, P)) {
-    int parts = 0;
-    FCK(f, project_gradient(f->dout, f->hp, f->wr + f->oQ2, f->dh, f->part, B, f->H, f->cout, P, f->sms, &parts, st));
+    const int parts = project_parts(B, P, f->sms);
     const long np = project_partials(f->H, f->cout);
+    if ((r = check_partials(f, (size_t)parts * np))) return r;
+    FCK(f, project_gradient(f->dout, f->hp, f->wr + f->oQ2, f->dh, f->part, B, f->H, f->cout, P, f->sms, st));
     FCK(f, sum_parts(f->part, np, parts, C * H, f->g + f->oQ2, st));
     FCK(f, sum_parts(f->part + C * H, np, parts, H, f->g + f->oq1, st));
     FCK(f, sum_parts(f->part + C * H + H, np, parts, C, f->g + f->oq2, st));

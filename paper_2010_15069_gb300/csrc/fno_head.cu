@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(kThreads, 1) map_points(const MapArgs a) {
 // dq1[c] = sum dhp[c] and dq2[o] = sum dout[o] stay in registers over the CTA's
 // tiles and leave as partials [CTA][cout H + H + cout].
 constexpr int kBackThreads = 512;
+static_assert(kHeadTile == kTcRows, "tiles of the projection");
 
 template <int H>
 __global__ void __launch_bounds__(kBackThreads, 1) project_backward(const float *__restrict__ dout,
@@ -373,12 +374,9 @@ cudaError_t project_transpose(const float *dhp, const void *q1w, float *dv, int 
   return width == 64 ? launch_map<128, 64, false>(a, sms, st) : launch_map<64, 32, false>(a, sms, st);
 }
 
-long project_partials(int hidden, int cout) { return (long)cout * hidden + hidden + cout; }
-
 cudaError_t project_gradient(const float *dout, const float *hp, const float *q2w, float *dhp, float *part, int batch,
-                             int hidden, int cout, long P, int sms, int *parts, cudaStream_t st) {
-  const int tpb = (int)(P / kTcRows), nt = batch * tpb, grid = std::max(1, std::min(nt, sms));
-  *parts = grid;
+                             int hidden, int cout, long P, int sms, cudaStream_t st) {
+  const int tpb = (int)(P / kTcRows), nt = batch * tpb, grid = project_parts(batch, P, sms);
   if (hidden == 128)
     project_backward<128><<<grid, kBackThreads, 0, st>>>(dout, hp, q2w, cout, nt, tpb, P, dhp, part);
   else

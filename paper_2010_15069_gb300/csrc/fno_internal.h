@@ -3,7 +3,9 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <vector>
 
@@ -71,8 +73,11 @@ struct WeightGrad {
   bool bias;
   int *flags;
 };
+constexpr long kGradBlock = 64;  // points per block of the MMA's K
 bool weight_grad_applies(const WeightGrad &g);
-int weight_grad_parts(int batch, long P, int sms);
+inline int weight_grad_parts(int batch, long P, int sms) {
+  return (int)std::max<long>(1, std::min<long>(2L * sms, batch * (P / kGradBlock)));
+}
 cudaError_t weight_grad(const WeightGrad &g, int sms, cudaStream_t st);
 cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool accumulate, cudaStream_t st);
 cudaError_t gemm_complex(const GemmC &g, cudaStream_t st);
@@ -104,21 +109,40 @@ cudaError_t layer_backward(const float *du, const float2 *G, const void *table, 
 // Lift and projection (fno_head.cu).  head_applies: W = 32 or 64 channels, 2 W
 // hidden ones, at most 4 outputs, P a multiple of 128.  project_forward: out =
 // Q2 gelu(Q1 v + q1) + q2, Q1 v + q1 to hp unless null.  project_gradient: dhp =
-// (Q2^T dout) gelu'(hp) and, per CTA (*parts of them), the sums dQ2 [cout][H],
-// dq1 [H], dq2 [cout] in project_partials() floats.  project_transpose: dv =
+// (Q2^T dout) gelu'(hp) and, per CTA (project_parts() of them), the sums dQ2
+// [cout][H], dq1 [H], dq2 [cout] in project_partials() floats.  project_transpose: dv =
 // Q1^T dhp.  lift_forward: v = A a + bias.
 bool head_applies(int width, int hidden, int cout, long P);
 cudaError_t project_forward(const float *v, const void *q1w, const float *q1b, const float *q2w, const float *q2b,
                             float *hp, float *out, int batch, int width, int cout, long P, int sms, int *flags,
                             cudaStream_t st);
-long project_partials(int hidden, int cout);
+constexpr long kHeadTile = 128;  // points per tile
+inline long project_partials(int hidden, int cout) { return (long)cout * hidden + hidden + cout; }
+inline int project_parts(int batch, long P, int sms) {
+  return (int)std::max<long>(1, std::min<long>(sms, batch * (P / kHeadTile)));
+}
 cudaError_t project_gradient(const float *dout, const float *hp, const float *q2w, float *dhp, float *part, int batch,
-                             int hidden, int cout, long P, int sms, int *parts, cudaStream_t st);
+                             int hidden, int cout, long P, int sms, cudaStream_t st);
 cudaError_t project_transpose(const float *dhp, const void *q1w, float *dv, int batch, int width, long P, int sms,
                               int *flags, cudaStream_t st);
 bool lift_applies(const float *in, int width, int cin, long P);
 cudaError_t lift_forward(const float *in, const float *w, const float *bias, float *v, int batch, int width, int cin,
                          long P, cudaStream_t st);
+// Floats that the partial sums of a network's weight gradients take, the largest
+// of: every product of weight and bias (M outputs, N inputs), per CTA on the
+// tensor cores or per split of `splits` in the general path, and the
+// projection's sums.
+inline int general_splits(long P) { return (int)std::max<long>(1, P / 1024); }
+inline size_t partial_floats(int cin, int cout, int width, int hidden, int batch, long P, int sms) {
+  const int shapes[4][2] = {{width, cin}, {width, width}, {hidden, width}, {cout, hidden}};
+  size_t most = (size_t)project_parts(batch, P, sms) * project_partials(hidden, cout);
+  for (const auto &q : shapes) {
+    const size_t mn = (size_t)q[0] * q[1];
+    most = std::max(most, (size_t)weight_grad_parts(batch, P, sms) * (mn + q[0]));
+    most = std::max(most, (size_t)batch * general_splits(P) * mn);
+  }
+  return most;
+}
 // out[i] = sum of part[k][i] over k < parts, in a fixed order; stride floats
 // from one part to the next.
 cudaError_t sum_parts(const float *part, long stride, int parts, long n, float *out, cudaStream_t st);

@@ -236,6 +236,7 @@ template <int MR, int NC> struct WgSmem {
 };
 
 constexpr int kWgThreads = 256;
+static_assert(kGradBlock == kKBlock, "a block of points is one K block");
 
 template <int MR, int NC>
 __global__ void __launch_bounds__(kWgThreads, 2) gemm_tc_wgrad(int M, int N, int nblk, int blocks_per_sample,
@@ -409,8 +410,6 @@ bool weight_grad_applies(const WeightGrad &g) {
   return g.M >= 1 && g.M <= 128 && g.N >= 1 && g.N <= 128 && g.P % kKBlock == 0 && g.sXb % 4 == 0 && g.sYb % 4 == 0 &&
          (reinterpret_cast<uintptr_t>(g.X) & 15) == 0 && (reinterpret_cast<uintptr_t>(g.Y) & 15) == 0;
 }
-
-int weight_grad_parts(int batch, long P, int sms) { return (int)std::max<long>(1, std::min<long>(2L * sms, batch * (P / kKBlock))); }
 
 cudaError_t weight_grad(const WeightGrad &g, int sms, cudaStream_t st) {
   const int grid = weight_grad_parts(g.batch, g.P, sms);
