@@ -39,6 +39,7 @@
 #include "async_copy.cuh"
 #include "fno_internal.h"
 #include "fno_umma.cuh"
+#include "internal.h"
 
 namespace spgpe {
 namespace fno {
@@ -493,8 +494,13 @@ cudaError_t dft_x(const float *v, const float *E, bool adjoint, float *X1, int i
 }
 
 cudaError_t dft_y(const float *X1, const float4 *Et, float2 *vh, int images, int n, int modes, cudaStream_t st) {
-  const int jt = (2 * modes + 3) / 4, per_block = std::max(1, kYThreads / (jt * (modes / 2)));
-  const size_t smem = (size_t)2 * kYBlock * (4 * jt * sizeof(float4) + per_block * modes * sizeof(float2));
+  // as many images as the threads cover and two buffers of kYBlock rows hold (two
+  // modes: 223 of 256, 232064 bytes; more modes are bounded by the threads)
+  const int jt = (2 * modes + 3) / 4;
+  const size_t table = 4 * jt * sizeof(float4), row = modes * sizeof(float2);  // of one y
+  const int fit = (int)((kMaxSmemPerBlock / (2 * kYBlock) - table) / row);
+  const int per_block = std::min(std::max(1, kYThreads / (jt * (modes / 2))), fit);
+  const size_t smem = 2 * kYBlock * (table + per_block * row);
   static size_t granted = 0;
   const cudaError_t e = grant(dft_cols, smem, granted);
   if (e != cudaSuccess) return e;
