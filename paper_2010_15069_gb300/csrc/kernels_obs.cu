@@ -11,6 +11,8 @@
 //    counter-based SplitMix64 stream (Sec. 6 annealing).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "fft_core.cuh"
 #include "internal.h"
 
@@ -18,8 +20,8 @@ namespace spgpe {
 
 namespace {
 
-template <int K> __device__ __forceinline__ void obs_block_sum(double (&v)[K]) {
-  __shared__ double red[K][32];
+// Block sum of v, valid in thread 0; red: K x 32 doubles of shared memory.
+template <int K> __device__ __forceinline__ void obs_block_sum(double (&v)[K], double (*red)[32]) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -117,12 +119,13 @@ __global__ void __launch_bounds__(256) sums_and_hist(const cx<T> *__restrict__ p
     }
     if (first && bin >= 0 && sum != 0.0) atomicAdd(&sh[bin], sum);
   }
-  obs_block_sum<4>(s);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 4; ++k) partials[((long)inst * gridDim.x + blockIdx.x) * 4 + k] = s[k];
   __syncthreads();
   for (int b = threadIdx.x; b < g.nb; b += blockDim.x)
     if (sh[b] != 0.0) atomicAdd(&hist[(long)inst * g.nb + b], sh[b]);
+  __syncthreads();  // the histogram is merged: its memory takes the sums
+  obs_block_sum<4>(s, reinterpret_cast<double(*)[32]>(sh));
+  if (threadIdx.x == 0)
+    for (int k = 0; k < 4; ++k) partials[((long)inst * gridDim.x + blockIdx.x) * 4 + k] = s[k];
 }
 
 template <class T> __device__ __forceinline__ double phase_at(const cx<T> *f, const ObsGeom &g, double x, double y) {
@@ -149,7 +152,7 @@ constexpr int kWindThreads = 256;
 template <class T>
 __global__ void __launch_bounds__(kWindThreads) winding(const cx<T> *__restrict__ psi, ObsGeom g, const double *R,
                                                         int npts, double *out) {
-  __shared__ double ph[kWindThreads + 1];
+  __shared__ double ph[kWindThreads + 1], red[1][32];
   const int comp = blockIdx.y, inst = blockIdx.z;
   const long plane = (long)g.nx * g.ny;
   const cx<T> *f = psi + ((long)inst * 2 + comp) * plane;
@@ -173,7 +176,7 @@ __global__ void __launch_bounds__(kWindThreads) winding(const cx<T> *__restrict_
     }
     __syncthreads();
   }
-  obs_block_sum<1>(s);
+  obs_block_sum<1>(s, red);
   if (threadIdx.x == 0) out[((long)inst * 2 + comp) * gridDim.x + blockIdx.x] = s[0];
 }
 
@@ -214,7 +217,9 @@ template <class T> cudaError_t obs_launch(const void *psi, const ObsGeom &g, int
   const cx<T> *p = reinterpret_cast<const cx<T> *>(psi);
   if (phase == 0) {
     const int rpb = (g.ny / 2 + sum_blocks - 1) / sum_blocks;  // pairs of mirrored rows
-    const size_t sm = (size_t)g.nb * sizeof(double);
+    // the histogram, or the sums after it; no other shared memory, so that up to
+    // 48 KB need no grant and kMaxSmemPerBlock bins of 8 bytes are the limit
+    const size_t sm = std::max((size_t)g.nb, (size_t)4 * 32) * sizeof(double);
     if (sm > 48 * 1024) {
       const cudaError_t e = cudaFuncSetAttribute(sums_and_hist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
