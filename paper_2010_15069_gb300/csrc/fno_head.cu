@@ -215,7 +215,8 @@ __global__ void __launch_bounds__(kThreads, 1) map_points(const MapArgs a) {
 // a tile of 128: dhp[b][c][p] = (sum_o Q2[o][c] dout[b][o][p]) gelu'(hp), in
 // place of hp or beside it; the sums dQ2[o][c] = sum dout[o] gelu(hp[c]),
 // dq1[c] = sum dhp[c] and dq2[o] = sum dout[o] stay in registers over the CTA's
-// tiles and leave as partials [CTA][cout H + H + cout].
+// tiles (one CTA per SM; more once they would exceed kHeadRun tiles each, which
+// keeps the float32 chains short) and leave as partials [CTA][cout H + H + cout].
 constexpr int kBackThreads = 512;
 static_assert(kHeadTile == kTcRows, "tiles of the projection");
 

@@ -73,10 +73,15 @@ struct WeightGrad {
   bool bias;
   int *flags;
 };
+// A CTA sums at most kGradRun blocks: the accumulator truncates, so its errors
+// have one sign and grow with the run (1024^2, batch 8: 5e-4 of a gradient in
+// runs of 431 blocks).
 constexpr long kGradBlock = 64;  // points per block of the MMA's K
+constexpr long kGradRun = 16;
 bool weight_grad_applies(const WeightGrad &g);
 inline int weight_grad_parts(int batch, long P, int sms) {
-  return (int)std::max<long>(1, std::min<long>(2L * sms, batch * (P / kGradBlock)));
+  const long blocks = batch * (P / kGradBlock);
+  return (int)std::max<long>(1, std::min(blocks, std::max(2L * sms, (blocks + kGradRun - 1) / kGradRun)));
 }
 cudaError_t weight_grad(const WeightGrad &g, int sms, cudaStream_t st);
 cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool accumulate, cudaStream_t st);
@@ -117,9 +122,11 @@ cudaError_t project_forward(const float *v, const void *q1w, const float *q1b, c
                             float *hp, float *out, int batch, int width, int cout, long P, int sms, int *flags,
                             cudaStream_t st);
 constexpr long kHeadTile = 128;  // points per tile
+constexpr long kHeadRun = 16;    // tiles whose float32 sums a CTA adds up at most
 inline long project_partials(int hidden, int cout) { return (long)cout * hidden + hidden + cout; }
 inline int project_parts(int batch, long P, int sms) {
-  return (int)std::max<long>(1, std::min<long>(sms, batch * (P / kHeadTile)));
+  const long tiles = batch * (P / kHeadTile);
+  return (int)std::max<long>(1, std::min(tiles, std::max<long>(sms, (tiles + kHeadRun - 1) / kHeadRun)));
 }
 cudaError_t project_gradient(const float *dout, const float *hp, const float *q2w, float *dhp, float *part, int batch,
                              int hidden, int cout, long P, int sms, cudaStream_t st);

@@ -224,10 +224,11 @@ cudaError_t launch_tc(const GemmR &g, cudaStream_t st) {
 // l l' is below 2^-16 of the result).  The MMA tile is 128 rows of X (M <= MR =
 // 64 or 128; the rows from M on stay zero) by NC = 16, 64 or 128 rows of Y (N <=
 // NC, likewise); the terms of Y lie side by side, so that X's h term meets both
-// in one MMA of 2 NC columns.  Persistent CTAs each take a run of 64-point
-// blocks and leave one partial sum; two operand buffers, the next block's
-// values in registers while the tensor cores work.  Bound by the one read of
-// both operands.
+// in one MMA of 2 NC columns.  A CTA takes a run of 64-point blocks and leaves
+// one partial sum: two CTAs per SM, and more of them once their runs would
+// exceed kGradRun blocks (the accumulator truncates, so its error grows with the
+// run); two operand buffers, the next block's values in registers while the
+// tensor cores work.  Bound by the one read of both operands.
 template <int MR, int NC> struct WgSmem {
   static constexpr size_t kA = (size_t)kTcRows * kRowBytes;  // one term of X
   static constexpr size_t kB = (size_t)NC * kRowBytes;       // one term of Y
