@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "fft_core.cuh"
 #include "fno_internal.h"
 
 namespace spgpe {
@@ -207,22 +208,23 @@ __global__ void reduce_splits(const float *__restrict__ part, long n, int splits
   }
 }
 
-// The same for few outputs and many parts: 8 threads per output, each every
-// eighth part, their sums added in order.
+// The same for few outputs and many parts, in FP64 (bias gradients, whose terms
+// cancel, lose no digits to the number of parts): 8 threads per output, each
+// every eighth part, their sums added in order.
 __global__ void __launch_bounds__(256) sum_parts_k(const float *__restrict__ part, long stride, int parts, long n,
                                                    float *out) {
-  __shared__ float red[8][33];
+  __shared__ double red[8][33];
   const int j = threadIdx.x & 31, s = threadIdx.x >> 5;
   const long i = (long)blockIdx.x * 32 + j;
-  float v = 0.f;
+  double v = 0.0;
   if (i < n)
-    for (int k = s; k < parts; k += 8) v += part[(long)k * stride + i];
+    for (int k = s; k < parts; k += 8) v += widen(part[(long)k * stride + i]);
   red[s][j] = v;
   __syncthreads();
   if (s == 0 && i < n) {
 #pragma unroll
     for (int q = 1; q < 8; ++q) v += red[q][j];
-    out[i] = v;
+    out[i] = (float)v;
   }
 }
 

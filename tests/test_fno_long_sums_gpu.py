@@ -67,3 +67,15 @@ def relative_errors(W, M, H, C):
 def test_weight_gradients_of_constant_fields(net):
     err = relative_errors(*net)
     assert all(err[k] < 3.1e-5 for k in ("Q2", "Q1", "W0")), err
+
+
+@pytest.mark.parametrize("net", NETS)
+def test_bias_gradients_of_constant_fields(net):
+    """16 additions of sums over 8 points (3) and 8 or 32 lanes (3 to 5), and up to 8
+    terms of the hidden gradient behind each value: 32 x 2^-24 = 2e-6; dw0 in addition
+    the 24 tensor-core steps of the transposed map: + 24 x 2^-23; the fused
+    projection's dQ2, 64 + 5 + 8 float32 steps: 4.6e-6."""
+    err = relative_errors(*net)
+    assert err["q2"] < 2e-6 and err["q1"] < 2e-6 and err["w0"] < 5e-6, err
+    if net[2] == 2 * net[0] and net[0] >= 32:
+        assert err["Q2"] < 4.6e-6, err
