@@ -74,6 +74,7 @@ struct spgpe_ctx {
   int tab_imag = -1;
   int omega_pieces = 0;
   double vbound2d = 0.0;  // max |V +- delta/2| of the 2D arrays (0 when separable)
+  std::vector<double> vabs, vmin, omax;  // per instance: max |V +- delta/2|, min of V +- delta/2, max |Omega|
   std::vector<double> h2d;  // host copy of the 2D {V + delta/2, V - delta/2, Omega, 0} table
   unsigned model_version = 0;
 
@@ -231,12 +232,19 @@ int upload_raw(spgpe_ctx *c) {
   r = upload(c, c->d_rawy, ry);
   if (r) return r;
   CK(c, cudaMemcpyAsync(c->d_gpar, c->hg.data(), c->hg.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
-  // Working-precision couplings {g11, g22, g12, Vb}, Vb = max |V +- delta/2| of
-  // the instance: the kernels bound the D phase with it to pick the small-phase
-  // series for a whole warp.
-  std::vector<double> gt(c->hg.size());
+  // Bounds of the potentials, for the kernels' choice of series (ensure_tables).
+  double v2min = 0.0, o2max = 0.0;
+  if (c->has2d) {
+    v2min = 1e300;
+    for (size_t k = 0; k < c->h2d.size(); k += 4) {
+      v2min = std::min(v2min, std::min(c->h2d[k], c->h2d[k + 1]));
+      o2max = std::max(o2max, std::fabs(c->h2d[k + 2]));
+    }
+  }
+  c->vabs.assign(c->ninst, 0.0);
+  c->vmin.assign(c->ninst, 1e300);
+  c->omax.assign(c->ninst, 0.0);
   for (int i = 0; i < c->ninst; ++i) {
-    double vb = 0.0;
     for (int sgn = -1; sgn <= 1; sgn += 2) {
       double xmin = 1e300, xmax = -1e300, ymin = 1e300, ymax = -1e300;
       for (int x = 0; x < c->nx; ++x) {
@@ -251,14 +259,15 @@ int upload_raw(spgpe_ctx *c) {
         ymin = std::min(ymin, v);
         ymax = std::max(ymax, v);
       }
-      vb = std::max(vb, std::max(std::fabs(xmin + ymin), std::fabs(xmax + ymax)));
+      c->vabs[i] = std::max(c->vabs[i], std::max(std::fabs(xmin + ymin), std::fabs(xmax + ymax)));
+      c->vmin[i] = std::min(c->vmin[i], xmin + ymin + v2min);
     }
-    gt[4 * i] = c->hg[4 * i];
-    gt[4 * i + 1] = c->hg[4 * i + 1];
-    gt[4 * i + 2] = c->hg[4 * i + 2];
-    gt[4 * i + 3] = vb + c->vbound2d;
+    double ox = 0.0, oy = 0.0;
+    for (int x = 0; x < c->nx; ++x) ox = std::max(ox, std::fabs(c->hx[((size_t)i * c->nx + x) * 3 + 2]));
+    for (int y = 0; y < c->ny; ++y) oy = std::max(oy, std::fabs(c->hy[((size_t)i * c->ny + y) * 3 + 2]));
+    c->vabs[i] += c->vbound2d;
+    c->omax[i] = ox + oy + o2max;
   }
-  if ((r = upload(c, c->d_gparT, gt))) return r;
   c->tab_dt = NAN;  // step tables depend on the model
   return SPGPE_OK;
 }
@@ -334,6 +343,23 @@ int ensure_tables(spgpe_ctx *c, double dt, int imag) {
     em1(dt * 0.5 * k * k, &ky[2 * (size_t)y]);
   }
   if (too_big) return fail(c, SPGPE_EINVAL, "|Omega| dt / 8 exceeds pi/2: time step too large for the Raman coupling");
+  // Working-precision couplings {g11, g22, g12, b}: the kernels bound the D
+  // exponent with b to pick the short series for a whole warp.  Real time: b =
+  // max |V +- delta/2|, the density at a point being constant.  Imaginary time: a
+  // bound of the density's growth within a pass, from where it is measured to
+  // the last D: three X (the opening one of R(dt/2) and the two between the two
+  // D of a fused pass), each exp(|Omega| dt / 8) in amplitude; the first D's
+  // potential factor exp(-(dt/2) V) where V is negative, and its interaction
+  // factor for attractive couplings, whose exponent a short series takes up to
+  // 1/2 (complex128 1/4).  At least 1.05, which covers the bound's own rounding.
+  std::vector<double> gt(c->hg);
+  for (int i = 0; i < ni; ++i) {
+    double *g = &gt[4 * (size_t)i];
+    const bool attract = g[0] < 0.0 || g[1] < 0.0 || g[2] < 0.0;
+    const double e = dt * (0.75 * c->omax[i] + std::max(0.0, -c->vmin[i])) +
+                     (attract ? (c->dtype == SPGPE_C64 ? 1.0 : 0.5) : 0.0);
+    g[3] = imag ? std::max(1.05, 1.001 * std::exp(std::min(e, 60.0))) : c->vabs[i];
+  }
   c->omega_pieces = 0;
   for (int i = 0; i < ni; ++i) {
     for (int y = 0; y < ny; ++y)
@@ -343,7 +369,7 @@ int ensure_tables(spgpe_ctx *c, double dt, int imag) {
   }
   int r;
   if ((r = upload(c, c->d_tabx, tx)) || (r = upload(c, c->d_taby, ty)) || (r = upload(c, c->d_kxt, kx)) ||
-      (r = upload(c, c->d_kyt, ky)))
+      (r = upload(c, c->d_kyt, ky)) || (r = upload(c, c->d_gparT, gt)))
     return r;
   c->tab_dt = dt;
   c->tab_imag = imag;

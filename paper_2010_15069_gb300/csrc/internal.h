@@ -46,7 +46,7 @@ struct RowArgs {
   const void *pot2d;      // [ny][nx] {V+delta/2, V-delta/2, Omega, 0} or null
   const void *tw;         // twiddle table of the x plan (see TwType in fft_core.cuh)
   const double *gpar;     // [ninst][4] {g11, g22, g12, kL}
-  const void *gparT;      // the same in the working precision
+  const void *gparT;      // {g11, g22, g12, b} in the working precision, b the bound of ensure_tables
   double tau;             // D substep (dt/2)
   double xang;            // X(dt/4) rotation angle per unit Omega (dt/8)
   double htau_d;          // -tau/2 (real time, half phase) or -tau (imaginary time)
