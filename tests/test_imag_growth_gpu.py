@@ -3,8 +3,10 @@ point where a pass bounds the interaction exponent and the factors that use
 it: the series that the bound picks must still hold.
 An antisymmetric spinor (the growing eigenvector of exp(-theta sigma_x)) whose
 exponent before the rotation lies just below each tier's bound, against the FP64
-oracle within the rounding of a few steps: complex128 1e-13 (entries below 1),
-complex64 the tolerance of its other step tests, 2e-6.
+oracle within the rounding of a step: complex128 1e-13 (entries below 1),
+complex64 the tolerance of its other step tests, 2e-6.  One step: where the peak is
+saturated and the tails grow by exp(5) a step, later steps amplify the transforms'
+rounding noise in the tails (twelvefold a step, the same in both precisions).
 """
 import numpy as np
 import pytest
@@ -33,7 +35,7 @@ def built():
 @pytest.mark.parametrize("target", [0.03, 0.24, 0.48])
 @pytest.mark.parametrize("omega,V0", [(1000.0, 0.0), (300.0, -200.0), (5.0, 0.0)])
 def test_growing_densities_match_the_oracle(orc, dtype, two_d, target, omega, V0):
-    n, box, dt, steps = 64, 8.0, 1e-2, 4
+    n, box, dt, steps = 64, 8.0, 1e-2, 1
     g = target / (0.5 * dt * 1.9 * 1.05 * 2 / np.pi)
     p = inputs.problem(n, n, box, box, Omega=omega, delta_slope=0.1, g11=g, g22=g, g12=0.9 * g, kL=0.5)
     u = inputs.gaussian_spinor(p.grid, width=1 / np.sqrt(2.0), noise=1e-2, seed=4)[0]
