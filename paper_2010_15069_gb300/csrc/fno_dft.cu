@@ -40,6 +40,7 @@
 #include "fno_internal.h"
 #include "fno_umma.cuh"
 #include "internal.h"
+#include "smem_grant.h"
 
 namespace spgpe {
 namespace fno {
@@ -391,22 +392,13 @@ __global__ void __launch_bounds__(kThreadsI, 2) idft_y(const IdftArgs a) {
   }
 }
 
-template <class K> cudaError_t grant(K kern, size_t smem, size_t &granted) {
-  if (smem > granted) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    granted = smem;
-  }
-  return cudaSuccess;
-}
-
 template <int CT>
 cudaError_t launch_rows(const float *v, const float *E, int n, int q2, float g0, float g1, float *out, long rows,
                         cudaStream_t st) {
   auto kern = dft_rows<CT>;
   constexpr size_t smem = (size_t)2 * (kXRows * kXStride + kXBlock * 8 * CT) * sizeof(float);
-  static size_t granted = 0;
-  const cudaError_t e = grant(kern, smem, granted);
+  static SmemGrant grant;
+  const cudaError_t e = grant(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)(rows / kXRows), 128, smem, st>>>(v, E, n, q2, g0, g1, out);
   return cudaGetLastError();
@@ -414,8 +406,8 @@ cudaError_t launch_rows(const float *v, const float *E, int n, int q2, float g0,
 
 template <int NY> cudaError_t launch_idft(const IdftArgs &a, int rows, cudaStream_t st) {
   auto kern = idft_y<NY>;
-  static size_t granted = 0;
-  const cudaError_t e = grant(kern, IdftSmem<NY>::kBytes, granted);
+  static SmemGrant grant;
+  const cudaError_t e = grant(kern, IdftSmem<NY>::kBytes);
   if (e != cudaSuccess) return e;
   kern<<<rows / kTcRows * a.ytiles, kThreadsI, IdftSmem<NY>::kBytes, st>>>(a);
   return cudaGetLastError();
@@ -501,8 +493,8 @@ cudaError_t dft_y(const float *X1, const float4 *Et, float2 *vh, int images, int
   const int fit = (int)((kMaxSmemPerBlock / (2 * kYBlock) - table) / row);
   const int per_block = std::min(std::max(1, kYThreads / (jt * (modes / 2))), fit);
   const size_t smem = 2 * kYBlock * (table + per_block * row);
-  static size_t granted = 0;
-  const cudaError_t e = grant(dft_cols, smem, granted);
+  static SmemGrant grant;
+  const cudaError_t e = grant(dft_cols, smem);
   if (e != cudaSuccess) return e;
   dft_cols<<<(unsigned)((images + per_block - 1) / per_block), kYThreads, smem, st>>>(reinterpret_cast<const float2 *>(X1), Et, n,
                                                                                modes, images, per_block, vh);

@@ -17,6 +17,7 @@
 #include "async_copy.cuh"
 #include "fno_internal.h"
 #include "fno_umma.cuh"
+#include "smem_grant.h"
 
 namespace spgpe {
 namespace fno {
@@ -343,12 +344,9 @@ template <int K, int N, bool PROJECT> cudaError_t launch_map(const MapArgs &a, i
   auto kern = map_points<K, N, PROJECT>;
   constexpr size_t smem = MapSmem<K, N>::kBytes;
   static_assert(smem <= 227 * 1024, "operand buffers within a block's limit");
-  static bool granted = false;
-  if (!granted) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    granted = true;
-  }
+  static SmemGrant grant;
+  const cudaError_t e = grant(kern, smem);
+  if (e != cudaSuccess) return e;
   kern<<<std::max(1, std::min(a.ntiles, sms)), kThreads, smem, st>>>(a);
   return cudaGetLastError();
 }

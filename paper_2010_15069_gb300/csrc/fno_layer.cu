@@ -32,6 +32,7 @@
 #include "async_copy.cuh"
 #include "fno_internal.h"
 #include "fno_umma.cuh"
+#include "smem_grant.h"
 
 namespace spgpe {
 namespace fno {
@@ -277,12 +278,9 @@ template <int W, int MODE> cudaError_t launch(const LayerArgs &a, int sms, cudaS
   auto kern = layer<W, MODE>;
   constexpr size_t smem = LayerSmem<W>::kBytes;
   static_assert(smem <= 227 * 1024, "operand buffers within a block's limit");
-  static bool granted = false;
-  if (!granted) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    granted = true;
-  }
+  static SmemGrant grant;
+  const cudaError_t e = grant(kern, smem);
+  if (e != cudaSuccess) return e;
   // every x tile has the same number of CTAs, at most one per row
   const int per = std::max(1, std::min(sms / a.xtiles, a.rows));
   kern<<<per * a.xtiles, kThreads, smem, st>>>(a);

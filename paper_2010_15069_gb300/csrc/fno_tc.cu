@@ -31,6 +31,7 @@
 #include "async_copy.cuh"
 #include "fno_internal.h"
 #include "fno_umma.cuh"
+#include "smem_grant.h"
 
 namespace spgpe {
 namespace fno {
@@ -197,16 +198,16 @@ template <int NC, int KB>
 cudaError_t launch_tc(const GemmR &g, cudaStream_t st) {
   auto kern = gemm_tc<NC, KB>;
   const size_t smem = TcSmem<NC, KB>::kBytes;
-  static int granted = 0, occ = 0, sms = 0;
-  if (!granted) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+  static SmemGrant grant;
+  cudaError_t e = grant(kern, smem);
+  if (e != cudaSuccess) return e;
+  static int occ = 0, sms = 0;
+  if (!sms) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 128, smem);
     if (e != cudaSuccess) return e;
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    granted = 1;
   }
   const int tpb = g.N / kTcRows, ntiles = tpb * g.batch;
   const int grid = std::max(1, std::min(ntiles, std::max(1, occ) * sms));
@@ -393,12 +394,9 @@ template <int MR, int NC>
 cudaError_t launch_wgrad(const WeightGrad &g, int grid, cudaStream_t st) {
   auto kern = gemm_tc_wgrad<MR, NC>;
   constexpr size_t smem = WgSmem<MR, NC>::kBytes;
-  static bool granted = false;
-  if (!granted) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    granted = true;
-  }
+  static SmemGrant grant;
+  const cudaError_t e = grant(kern, smem);
+  if (e != cudaSuccess) return e;
   const int bps = (int)(g.P / kKBlock);
   kern<<<grid, kWgThreads, smem, st>>>(g.M, g.N, g.batch * bps, bps, g.X, g.P, g.sXb, g.Y, g.P, g.sYb, g.part,
                                        (long)g.M * g.N + (g.bias ? g.M : 0), g.bias ? 1 : 0, g.flags);

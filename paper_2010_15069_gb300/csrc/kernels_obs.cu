@@ -15,6 +15,7 @@
 
 #include "fft_core.cuh"
 #include "internal.h"
+#include "smem_grant.h"
 
 namespace spgpe {
 
@@ -220,10 +221,9 @@ template <class T> cudaError_t obs_launch(const void *psi, const ObsGeom &g, int
     // the histogram, or the sums after it; no other shared memory, so that up to
     // 48 KB need no grant and kMaxSmemPerBlock bins of 8 bytes are the limit
     const size_t sm = std::max((size_t)g.nb, (size_t)4 * 32) * sizeof(double);
-    if (sm > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(sums_and_hist<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e != cudaSuccess) return e;
-    }
+    static SmemGrant grant;
+    const cudaError_t e = sm > 48 * 1024 ? grant(sums_and_hist<T>, sm) : cudaSuccess;
+    if (e != cudaSuccess) return e;
     sums_and_hist<T><<<dim3(sum_blocks, ninst), 256, sm, st>>>(p, g, rpb, partials, hist);
   } else {
     winding<T><<<dim3(kWindBlocks, 2, ninst), kWindThreads, 0, st>>>(p, g, R, npts, wind);

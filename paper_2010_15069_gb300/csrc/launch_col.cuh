@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "kernels_persist.cuh"
+#include "smem_grant.h"
 
 namespace spgpe {
 
@@ -23,15 +24,6 @@ template <class T> LaunchShape col_shape(int nx, int ny) {
   s.rows_or_cols = C;
   s.smem = (size_t)col_smem_elems(ny, C, sizeof(cx<T>)) * sizeof(cx<T>);
   return s;
-}
-
-template <class K> cudaError_t grant_smem_c(K kern, size_t smem, int &granted) {
-  if ((int)smem > granted) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    granted = (int)smem;
-  }
-  return cudaSuccess;
 }
 
 // Columns per block of the plain column pass for a batch of ninst instances:
@@ -56,8 +48,8 @@ template <class T, int LOGN, bool IMAG> cudaError_t col_launch_n(ColArgs a, cuda
   constexpr int LOGE = col_loge<T>(LOGN);
   auto kern = col_pass<T, LOGN, LOGE, IMAG>;
   const LaunchShape sh = col_shape_spread<T>(a.nx, a.ny, a.ninst, sms);
-  static int granted = 0;
-  cudaError_t e = grant_smem_c(kern, sh.smem, granted);
+  static SmemGrant grant;
+  cudaError_t e = grant(kern, sh.smem);
   if (e != cudaSuccess) return e;
   a.C = sh.rows_or_cols;
   a.pdl_early = a.overlap && sizeof(T) == 4 && (long)sh.blocks_x * 2 * a.ninst <= sms;
@@ -73,8 +65,8 @@ template <class T, int LOGN> cudaError_t energy_launch_n(EnergyArgs a, cudaStrea
     const int TT = a.nx / E;
     const int rows = std::max(1, std::min(kRowMaxThreads / TT, a.ny));
     const size_t smem = (size_t)rows * row_stride(a.nx, sizeof(cx<T>)) * sizeof(cx<T>);
-    static int granted = 0;
-    cudaError_t e = grant_smem_c(kern, smem, granted);
+    static SmemGrant grant;
+    cudaError_t e = grant(kern, smem);
     if (e != cudaSuccess) return e;
     a.rows = rows;
     *rb = a.ny / rows;
@@ -89,8 +81,8 @@ template <class T, int LOGN> cudaError_t energy_col_launch_n(EnergyArgs a, cudaS
   constexpr int LOGE = col_loge<T>(LOGN);
   auto kern = energy_col<T, LOGN, LOGE>;
   const LaunchShape sh = col_shape<T>(a.nx, a.ny);
-  static int granted = 0;
-  cudaError_t e = grant_smem_c(kern, sh.smem, granted);
+  static SmemGrant grant;
+  cudaError_t e = grant(kern, sh.smem);
   if (e != cudaSuccess) return e;
   a.C = sh.rows_or_cols;
   *cb = sh.blocks_x;
@@ -183,8 +175,8 @@ cudaError_t colp_launch_n(ColArgs a, const CUtensorMap &map, cudaStream_t st, in
   const size_t smem = kPipe * colp_buf_bytes(N, C, es) + (size_t)N * es +
                       colp_tw_bytes<T>(LOGN, C, Plan<LOGN, LOGE>::entries()) + kPipe * sizeof(uint64_t);
   if (smem > kMaxSmemPerBlock) return cudaErrorNotSupported;  // caller falls back to the plain pass
-  static int granted = 0;
-  cudaError_t e = grant_smem_c(kern, smem, granted);
+  static SmemGrant grant;
+  cudaError_t e = grant(kern, smem);
   if (e != cudaSuccess) return e;
   static int occ_threads = -1, occ_blocks = 0;
   static size_t occ_smem = 0;
@@ -219,8 +211,9 @@ template <class T> cudaError_t launch_col_p(bool imag, ColArgs a, const CUtensor
 template <bool IMAG> cudaError_t colw_launch(ColArgs a, const CUtensorMap &map, cudaStream_t st, int sms) {
   auto kern = col_pass_w<IMAG>;
   const size_t smem = colw_smem();
-  static int granted = 0, occ = -1;  // per instantiation (per time direction)
-  cudaError_t e = grant_smem_c(kern, smem, granted);
+  static SmemGrant grant;
+  static int occ = -1;  // per instantiation (per time direction)
+  cudaError_t e = grant(kern, smem);
   if (e != cudaSuccess) return e;
   if (occ < 0 && (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, smem)) != cudaSuccess) return e;
   const int ntiles = (a.nx / kColW_C) * 2 * a.ninst;

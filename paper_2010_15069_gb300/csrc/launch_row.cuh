@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "kernels_persist.cuh"
+#include "smem_grant.h"
 
 namespace spgpe {
 
@@ -24,25 +25,13 @@ template <class T> LaunchShape row_shape(int nx, int ny) {
   return s;
 }
 
-template <class K> cudaError_t grant_smem(K kern, size_t smem, int &granted) {
-  if ((int)smem > granted) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    granted = (int)smem;
-  }
-  return cudaSuccess;
-}
-
 template <class T, int LOGN, int F> cudaError_t row_launch_n(RowArgs a, cudaStream_t st) {
   constexpr int LOGE = row_loge<T>(LOGN);
   auto kern = row_pass<T, LOGN, LOGE, F>;
   const LaunchShape sh = row_shape<T>(a.nx, a.ny);
-  static int attr_set = 0;  // largest dynamic shared memory granted so far
-  if ((int)sh.smem > attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
-    if (e != cudaSuccess) return e;
-    attr_set = (int)sh.smem;
-  }
+  static SmemGrant grant;
+  const cudaError_t e = grant(kern, sh.smem);
+  if (e != cudaSuccess) return e;
   a.rows = sh.rows_or_cols;
   return launch_pdl(a.overlap, kern, dim3(sh.blocks_x, a.ninst), sh.threads, sh.smem, st, a);
 }
@@ -86,8 +75,8 @@ template <class T, int LOGN, int F> cudaError_t rowp_launch_n(RowArgs a, cudaStr
   const size_t full_smem = rowu_smem(N, E, sizeof(cx<T>), Plan<LOGN, LOGE>::entries());
   const size_t smem = U::WARP ? full_smem - (size_t)(most - upb) * rowu_bytes(N, U::ROWS, sizeof(cx<T>)) : full_smem;
   if (full_smem > kMaxSmemPerBlock) return cudaErrorNotSupported;
-  static int granted = 0;
-  cudaError_t e = grant_smem(kern, full_smem, granted);  // (a full block's, which the occupancy below is asked for)
+  static SmemGrant grant;
+  cudaError_t e = grant(kern, full_smem);  // (a full block's, which the occupancy below is asked for)
   if (e != cudaSuccess) return e;
   static int occ_blocks = -1;  // of full blocks (a smaller one is not launched more than once per SM)
   if (occ_blocks < 0) {
