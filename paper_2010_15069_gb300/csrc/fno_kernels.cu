@@ -12,7 +12,6 @@
 #include <algorithm>
 #include <cmath>
 
-#include "fft_core.cuh"
 #include "fno_internal.h"
 
 namespace spgpe {
@@ -208,23 +207,45 @@ __global__ void reduce_splits(const float *__restrict__ part, long n, int splits
   }
 }
 
-// The same for few outputs and many parts, in FP64 (bias gradients, whose terms
-// cancel, lose no digits to the number of parts): 8 threads per output, each
-// every eighth part, their sums added in order.
+// A float32 sum with its rounding errors summed beside it (Knuth's two-sum): the
+// digits of an FP64 sum for six float32 additions per term, which GB300 does at
+// more than ten times the rate of one FP64 addition.
+struct Sum2 {
+  float hi, lo;
+  __device__ __forceinline__ void add(float x) {
+    const float t = __fadd_rn(hi, x), u = __fsub_rn(t, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, u)), __fsub_rn(x, u)));
+    hi = t;
+  }
+  __device__ __forceinline__ void add(const Sum2 &o) {
+    add(o.hi);
+    lo = __fadd_rn(lo, o.lo);
+  }
+  __device__ __forceinline__ float value() const { return lo == lo ? __fadd_rn(hi, lo) : hi; }  // (an infinite sum stays one)
+};
+
+// The same for few outputs and many parts: bias gradients, whose terms cancel,
+// lose no digits to the number of parts.  Bound by the latency of the reads: 32
+// threads per output, each every 32nd part, 8 outputs (a sector) per block, the
+// threads' sums added in a fixed tree.  A training step at 256^2, batch 4 (14
+// calls, 304 parts): 56 us; float32 sums by 8 threads each 87 us, FP64 133 us.
 __global__ void __launch_bounds__(256) sum_parts_k(const float *__restrict__ part, long stride, int parts, long n,
                                                    float *out) {
-  __shared__ double red[8][33];
-  const int j = threadIdx.x & 31, s = threadIdx.x >> 5;
-  const long i = (long)blockIdx.x * 32 + j;
-  double v = 0.0;
+  __shared__ Sum2 red[8][8];
+  const int j = threadIdx.x & 7, s = threadIdx.x >> 3, w = threadIdx.x >> 5;
+  const long i = (long)blockIdx.x * 8 + j;
+  Sum2 v{0.f, 0.f};
   if (i < n)
-    for (int k = s; k < parts; k += 8) v += widen(part[(long)k * stride + i]);
-  red[s][j] = v;
-  __syncthreads();
-  if (s == 0 && i < n) {
+    for (int k = s; k < parts; k += 32) v.add(part[(long)k * stride + i]);
 #pragma unroll
-    for (int q = 1; q < 8; ++q) v += red[q][j];
-    out[i] = (float)v;
+  for (int o = 8; o < 32; o <<= 1)
+    v.add(Sum2{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+  if ((threadIdx.x & 31) < 8) red[w][j] = v;
+  __syncthreads();
+  if (threadIdx.x < 8 && i < n) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) v.add(red[q][j]);
+    out[i] = v.value();
   }
 }
 
@@ -484,7 +505,7 @@ cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool a
 }
 
 cudaError_t sum_parts(const float *part, long stride, int parts, long n, float *out, cudaStream_t st) {
-  sum_parts_k<<<(unsigned)((n + 31) / 32), 256, 0, st>>>(part, stride, parts, n, out);
+  sum_parts_k<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(part, stride, parts, n, out);
   return cudaGetLastError();
 }
 
