@@ -281,7 +281,7 @@ __device__ __forceinline__ double expm1_small(double x) {  // |x| < 1/4
   p = fma(x, p, 0.5);
   return fma(x * x, p, x);
 }
-__device__ __forceinline__ double expm1_quarter(double x) {  // |x| < 1/32 (the first tier in double precision)
+__device__ __forceinline__ double expm1_32nd(double x) {  // |x| < 1/32
   double p = fma(x, 1.0 / 362880.0, 1.0 / 40320.0);
   p = fma(x, p, 1.0 / 5040.0);
   p = fma(x, p, 1.0 / 720.0);

@@ -20,11 +20,6 @@ namespace {
 
 const double kTwoPi = 6.28318530717958647692528676655900577;
 
-struct Buf {
-  float *p = nullptr;
-  size_t n = 0;
-};
-
 }  // namespace
 
 struct spgpe_fno {
@@ -212,8 +207,7 @@ GemmR rg(int M, int N, int K, const void *A, bool bf, long sAm, long sAk, const 
 }
 
 GemmC cg(int M, int N, int K, int batch, const void *A, bool bf, bool ca, long sAm, long sAk, long sAb,
-         const float2 *Bm, bool cb, long sBk, long sBn, long sBb, float2 *C, long sCm, long sCn, long sCb,
-         float beta = 0.f) {
+         const float2 *Bm, bool cb, long sBk, long sBn, long sBb, float2 *C, long sCm, long sCn, long sCb) {
   GemmC g;
   g.M = M;
   g.N = N;
@@ -234,7 +228,6 @@ GemmC cg(int M, int N, int K, int batch, const void *A, bool bf, bool ca, long s
   g.sCm = sCm;
   g.sCn = sCn;
   g.sCb = sCb;
-  g.beta = beta;
   return g;
 }
 
@@ -286,7 +279,7 @@ int wgrad(spgpe_fno *f, int M, int N, long P, int B, const float *A, long sAb, c
   g.partial = true;
   g.sCs = (long)M * N;
   FCK(f, greal(f, g, f->st));
-  FCK(f, sum_splits(f->part, (long)M * N, B * splits, grad, false, f->st));
+  FCK(f, sum_splits(f->part, (long)M * N, B * splits, grad, f->st));
   if (bias) FCK(f, bias_gradient(A, B, M, P, bias, f->bscr, f->st));
   return SPGPE_OK;
 }

@@ -1,5 +1,7 @@
-// Launchers of the Fourier-neural-operator kernels (fno_kernels.cu), used by
-// the C ABI in fno.cu.
+// Launchers of the Fourier-neural-operator kernels, used by the C ABI in fno.cu:
+// general products and reductions (fno_kernels.cu), tensor-core channel maps and
+// weight gradients (fno_tc.cu), transforms (fno_dft.cu), layers (fno_layer.cu),
+// mode mixing (fno_mix.cu), lift and projection (fno_head.cu).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -34,12 +36,10 @@ struct GemmR {
   int *flags = nullptr;
 };
 
-// Complex C(m, n) = sum_k op(A)(m, k) op(B)(k, n) + beta C(m, n), strides in
-// complex elements; op conjugates when conj_a / conj_b (not both); A may be
+// Complex C(m, n) = sum_k op(A)(m, k) op(B)(k, n), strides in complex elements; op conjugates when conj_a / conj_b (not both); A may be
 // bfloat16 pairs (a_bf16; then not conjugated).
 struct GemmC {
   int M, N, K, batch = 1;
-  float beta = 0.f;
   const void *A;
   bool a_bf16 = false, conj_a = false, conj_b = false;
   long sAm, sAk, sAb = 0;
@@ -84,7 +84,7 @@ inline int weight_grad_parts(int batch, long P, int sms) {
   return (int)std::max<long>(1, std::min(blocks, std::max(2L * sms, (blocks + kGradRun - 1) / kGradRun)));
 }
 cudaError_t weight_grad(const WeightGrad &g, int sms, cudaStream_t st);
-cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool accumulate, cudaStream_t st);
+cudaError_t sum_splits(const float *part, long n, int splits, float *out, cudaStream_t st);
 cudaError_t gemm_complex(const GemmC &g, cudaStream_t st);
 // Truncated Fourier transforms (fno_dft.cu) of `images` n x n fields with the
 // kept modes kx < M, ky = -M .. M - 1 (M even, at most 32; n a multiple of 64;

@@ -198,10 +198,10 @@ __global__ void __launch_bounds__(256) gemm_r2(int M, int N, int K, int splits, 
   }
 }
 
-// out[i] (+)= sum_s part[s][i] in the order s = 0, 1, ...
-__global__ void reduce_splits(const float *__restrict__ part, long n, int splits, float *out, int accumulate) {
+// out[i] = sum_s part[s][i] in the order s = 0, 1, ...
+__global__ void reduce_splits(const float *__restrict__ part, long n, int splits, float *out) {
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    float s = accumulate ? out[i] : 0.f;
+    float s = 0.f;
     for (int k = 0; k < splits; ++k) s += part[(long)k * n + i];
     out[i] = s;
   }
@@ -263,7 +263,7 @@ __device__ __forceinline__ c2 ld_c(const __nv_bfloat162 *p) {
 template <class TA, bool CA, bool CB>
 __global__ void __launch_bounds__(256) gemm_c(int M, int N, int K, const TA *__restrict__ A, long sAm, long sAk,
                                               long sAb, const float2 *__restrict__ B, long sBk, long sBn, long sBb,
-                                              float beta, float2 *C, long sCm, long sCn, long sCb) {
+                                              float2 *C, long sCm, long sCn, long sCb) {
   __shared__ c2 As[TK][TM + 1];
   __shared__ c2 Bs[TK][TN + 1];
   const int bt = blockIdx.z;
@@ -316,14 +316,7 @@ __global__ void __launch_bounds__(256) gemm_c(int M, int N, int K, const TA *__r
     for (int j = 0; j < 4; ++j) {
       const int gn = n0 + tx + 16 * j;
       if (gn >= N) continue;
-      float2 *c = C + gm * sCm + gn * sCn;
-      float2 v = make_float2(acc[i][j].x, acc[i][j].y);
-      if (beta != 0.f) {
-        const float2 o = *c;
-        v.x = fmaf(beta, o.x, v.x);
-        v.y = fmaf(beta, o.y, v.y);
-      }
-      *c = v;
+      C[gm * sCm + gn * sCn] = make_float2(acc[i][j].x, acc[i][j].y);
     }
   }
 }
@@ -499,8 +492,8 @@ cudaError_t gemm_real(const GemmR &g, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t sum_splits(const float *part, long n, int splits, float *out, bool accumulate, cudaStream_t st) {
-  reduce_splits<<<grid_for(n), 256, 0, st>>>(part, n, splits, out, accumulate ? 1 : 0);
+cudaError_t sum_splits(const float *part, long n, int splits, float *out, cudaStream_t st) {
+  reduce_splits<<<grid_for(n), 256, 0, st>>>(part, n, splits, out);
   return cudaGetLastError();
 }
 
@@ -513,7 +506,7 @@ cudaError_t gemm_complex(const GemmC &g, cudaStream_t st) {
   const dim3 grid((g.N + TN - 1) / TN, (g.M + TM - 1) / TM, g.batch);
 #define SPGPE_GC(TA, CA, CB)                                                                                    \
   gemm_c<TA, CA, CB><<<grid, 256, 0, st>>>(g.M, g.N, g.K, static_cast<const TA *>(g.A), g.sAm, g.sAk, g.sAb, g.B, \
-                                           g.sBk, g.sBn, g.sBb, g.beta, g.C, g.sCm, g.sCn, g.sCb)
+                                           g.sBk, g.sBn, g.sBb, g.C, g.sCm, g.sCn, g.sCb)
   if (g.a_bf16) {
     if (g.conj_a) SPGPE_GC(__nv_bfloat162, true, false);
     else SPGPE_GC(__nv_bfloat162, false, false);

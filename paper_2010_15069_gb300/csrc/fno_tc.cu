@@ -247,17 +247,15 @@ __global__ void __launch_bounds__(kWgThreads, 2) gemm_tc_wgrad(int M, int N, int
                                                             long sPs, int with_bias, int *flags) {
   using S = WgSmem<MR, NC>;
   constexpr uint32_t kCols = 2 * NC < 32 ? 32 : 2 * NC;
-  constexpr int CH = (MR + NC) * 8 / kWgThreads;  // 16-byte runs of one 64-point block per thread
-  constexpr int CHX = MR * 8 / kWgThreads;        // those of X
+  constexpr int CHX = MR * 8 / kWgThreads;  // 16-byte runs of X of one 64-point block per thread
   static_assert((MR + NC) * 8 % kWgThreads == 0 || NC == 16, "whole runs per thread");
-  constexpr int CHT = ((MR + NC) * 8 + kWgThreads - 1) / kWgThreads;
+  constexpr int CHT = ((MR + NC) * 8 + kWgThreads - 1) / kWgThreads;  // those of X and Y
   extern __shared__ unsigned char smem_raw[];
   unsigned char *sm =
       reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t *mma = reinterpret_cast<uint64_t *>(sm + 2 * S::kStage);
   uint32_t *slot = reinterpret_cast<uint32_t *>(mma + 2);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  (void)CH;
   const int b0 = (int)((long)blockIdx.x * nblk / gridDim.x), b1 = (int)((long)(blockIdx.x + 1) * nblk / gridDim.x);
 
   if (warp == 0) {

@@ -1,7 +1,8 @@
 // tcgen05 building blocks shared by the Fourier neural operator's tensor-core
-// kernels (fno_tc.cu, fno_spectral.cu): K-major bfloat16 operands in shared
-// memory with the 128-byte swizzle, MMA issue and commit, tensor-memory
-// allocation and loads, and the split of float32 values into bfloat16 terms.
+// kernels (fno_tc.cu, fno_dft.cu, fno_layer.cu, fno_head.cu): K-major bfloat16
+// operands in shared memory with the 128-byte swizzle, MMA issue and commit,
+// tensor-memory allocation and loads, and the split of float32 values into
+// bfloat16 terms.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

@@ -178,10 +178,10 @@ struct ObsGeom {
   double xmax, ymax, dx, dy, h;
 };
 // phase 0: FP64 sums {rho_up rho_dn, rho_up^2, rho_dn^2, rho_up + rho_dn} per
-// block and instance into partials ([ninst][sum_blocks][4]) and the radial histogram of the total density into hist ([ninst][nb],
-// zeroed by the caller); phase 1: phase steps around radius R[inst] with npts
-// points, summed per block into wind ([ninst][2][kWindBlocks]).  es = bytes per
-// complex element.
+// block and instance into partials ([ninst][sum_blocks][4]) and the radial
+// histogram of the total density into hist ([ninst][nb], zeroed by the caller);
+// phase 1: phase steps around radius R[inst] with npts points, summed per block
+// into wind ([ninst][2][kWindBlocks]).  es = bytes per complex element.
 constexpr int kWindBlocks = 8;
 cudaError_t launch_observables(int es, const void *psi, const ObsGeom &g, int ninst, double *partials,
                                int sum_blocks, double *hist, const double *R, int npts, double *wind, int phase,

@@ -118,8 +118,13 @@ __device__ __forceinline__ void opD(cx<T> &u, cx<T> &d, T vu, T vd, T gh11, T gh
     const T hu = d_fma(gh12, rd, gh11 * ru), hd = d_fma(gh12, ru, gh22 * rd);
     T fu, fd;
     if constexpr (TIER == 0) {
-      fu = expm1_quarter(hu);
-      fd = expm1_quarter(hd);
+      if constexpr (sizeof(T) == 4) {
+        fu = expm1_quarter(hu);
+        fd = expm1_quarter(hd);
+      } else {
+        fu = expm1_32nd(hu);
+        fd = expm1_32nd(hd);
+      }
     } else if constexpr (TIER == 1) {
       fu = expm1_small(hu);
       fd = expm1_small(hd);
