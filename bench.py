@@ -667,7 +667,7 @@ def fno_throughput(n=256, batch=4, steps=10):
                         "bfloat16 weights, FP32 accumulate, one Adam step per batch",
             "ms_per_train_step": sec * 1e3, "samples_per_s": batch / sec,
             "achieved_tflops": flop / sec / 1e12,
-            "where": "channel products and weight gradients on tcgen05 tensor cores; truncated DFTs and mode "
+            "where": "channel maps, inverse DFTs and weight gradients on tcgen05 tensor cores; forward DFTs and mode "
                      "mixing on CUDA cores"}
 
 
