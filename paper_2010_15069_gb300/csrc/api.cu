@@ -345,20 +345,27 @@ int ensure_tables(spgpe_ctx *c, double dt, int imag) {
   if (too_big) return fail(c, SPGPE_EINVAL, "|Omega| dt / 8 exceeds pi/2: time step too large for the Raman coupling");
   // Working-precision couplings {g11, g22, g12, b}: the kernels bound the D
   // exponent with b to pick the short series for a whole warp.  Real time: b =
-  // max |V +- delta/2|, the density at a point being constant.  Imaginary time: a
-  // bound of the density's growth within a pass, from where it is measured to
-  // the last D: three X (the opening one of R(dt/2) and the two between the two
-  // D of a fused pass), each exp(|Omega| dt / 8) in amplitude; the first D's
-  // potential factor exp(-(dt/2) V) where V is negative, and its interaction
-  // factor for attractive couplings, whose exponent a short series takes up to
-  // 1/2 (complex128 1/4).  At least 1.05, which covers the bound's own rounding.
+  // max |V +- delta/2|, the density at a point being constant.  Imaginary time: b
+  // = max(|g11|, |g22|) + |g12| (in the working precision) times a bound of the
+  // density's growth within a pass, from where it is measured to the last D:
+  // three X (the opening one of R(dt/2) and the two between the two D of a fused
+  // pass), each exp(|Omega| dt / 8) in amplitude; the first D's potential factor
+  // exp(-(dt/2) V) where V is negative, and its interaction factor for attractive
+  // couplings, whose exponent a short series takes up to 1/2 (complex128 1/4).  At
+  // least 1.05, which covers the bound's own rounding.
   std::vector<double> gt(c->hg);
   for (int i = 0; i < ni; ++i) {
     double *g = &gt[4 * (size_t)i];
     const bool attract = g[0] < 0.0 || g[1] < 0.0 || g[2] < 0.0;
     const double e = dt * (0.75 * c->omax[i] + std::max(0.0, -c->vmin[i])) +
                      (attract ? (c->dtype == SPGPE_C64 ? 1.0 : 0.5) : 0.0);
-    g[3] = imag ? std::max(1.05, 1.001 * std::exp(std::min(e, 60.0))) : c->vabs[i];
+    const double grow = std::max(1.05, 1.001 * std::exp(std::min(e, 60.0)));
+    if (!imag)
+      g[3] = c->vabs[i];
+    else if (c->dtype == SPGPE_C64)
+      g[3] = (std::max(std::fabs((float)g[0]), std::fabs((float)g[1])) + std::fabs((float)g[2])) * (float)grow;
+    else
+      g[3] = (std::max(std::fabs(g[0]), std::fabs(g[1])) + std::fabs(g[2])) * grow;
   }
   c->omega_pieces = 0;
   for (int i = 0; i < ni; ++i) {

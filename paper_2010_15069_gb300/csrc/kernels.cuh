@@ -448,10 +448,10 @@ __device__ __forceinline__ void r_apply(cx<T> (&pu)[K], cx<T> (&pd)[K], int t, i
   // rho_tot with Vb = max |V +- delta/2| of the instance (gp[3]) and G = max(|g11|,
   // |g22|) + |g12|; R leaves rho_tot = |u|^2 + |d|^2 at a point unchanged (5 %
   // margin for rounding).  Imaginary time: the potential factors come from
-  // tables, so only the interaction exponent is bounded, with the density's
-  // growth up to the last D in gp[3]; the lagged pass also scales the densities
-  // between R_end and R_start by the squared predicted scale.  Double precision
-  // bounds it in single precision, with the magnitudes from integer
+  // tables, so only the interaction exponent is bounded, with G times the
+  // density's growth up to the last D in gp[3]; the lagged pass also scales the
+  // densities between R_end and R_start by the squared predicted scale.  Double
+  // precision bounds it in single precision, with the magnitudes from integer
   // instructions: the margins cover the rounding.
   float hb;
   if constexpr (sizeof(T) == 4) {
@@ -460,7 +460,7 @@ __device__ __forceinline__ void r_apply(cx<T> (&pu)[K], cx<T> (&pd)[K], int t, i
     for (int j = 0; j < K; ++j) rmax = fmax(rmax, d_fma(pu[j].re, pu[j].re, pu[j].im * pu[j].im) +
                                                       d_fma(pd[j].re, pd[j].re, pd[j].im * pd[j].im));
     if constexpr ((F & F_LAG) != 0) rmax *= fmax(T(1), fmax(su * su, sd * sd));
-    hb = fabs(htau) * (IMAG ? gmax * gp[3] * rmax : gp[3] + gmax * T(1.05) * rmax);
+    hb = fabs(htau) * (IMAG ? gp[3] * rmax : gp[3] + gmax * T(1.05) * rmax);
   } else {
     float rmax = 0.f;
 #pragma unroll
@@ -472,8 +472,8 @@ __device__ __forceinline__ void r_apply(cx<T> (&pu)[K], cx<T> (&pd)[K], int t, i
       const float fu = magnitude_f(su), fd = magnitude_f(sd);
       rmax *= fmaxf(1.f, fmaxf(fu * fu, fd * fd) * 1.00001f);
     }
-    const float b = magnitude_f(gp[3]) * 1.00001f, gm = magnitude_f(gmax);
-    hb = magnitude_f(htau) * 1.00001f * (IMAG ? gm * b * rmax : b + gm * 1.05f * rmax);
+    const float b = magnitude_f(gp[3]) * 1.00001f;
+    hb = magnitude_f(htau) * 1.00001f * (IMAG ? b * rmax : b + magnitude_f(gmax) * 1.05f * rmax);
     if (!(rmax < 1e30f)) hb = 1e30f;  // not finite: fmaxf drops a NaN, the library functions pass it on
   }
   constexpr float kSmall = IMAG ? (sizeof(T) == 4 ? 0.5f : 0.25f) : 0.125f;
